@@ -5,6 +5,8 @@
 #include <cudaTypedefs.h>
 #include <stdint.h>
 
+#include <vector>
+
 #include "../../include/vamrt.h"
 
 namespace vamrt {
@@ -42,6 +44,22 @@ struct OpParams {
     float y0;             // start of chunk 0 on the theta = 0 frame's y axis, voxels
     float cell_bound;     // most samples of one ray whose footprint holds a given voxel
     float h_over_m;       // voxel pitch (mm) / rays per pixel: delta_mm / M = delta_vox * h_over_m
+};
+
+// Per-launch constants of the grouped operators (ring.cuh).  Groups of S angles a quarter,
+// half or whole turn apart are walked together on rotated copies of the volume.
+struct RingParams {
+    OpParams op;
+    int n_groups;
+    const double2 *cs;     // (cos, sin) of each group's first angle, FP64
+    const int *members;    // S angle indices per group, 2 pi / S apart
+    int pzp;               // z extent of the rotated copies: nz + 2 rounded up to 4
+    int64_t vol_elems;     // voxels of one copy: (nx + 2) (ny + 2) pzp
+    const unsigned char *bricks;   // occupancy of the rotated copies, 8^3 voxels a byte
+    int bzp;               // bricks along z, rounded up to 8
+    int64_t brick_stride;  // bricks of one copy
+    const CUtensorMap *maps;   // device: [copy][EX class][EZ class]
+    int n_ex;              // EX classes
 };
 
 // Per-ray constants of the FP64 tracer.
@@ -83,6 +101,13 @@ struct vamrt_projector {
     float *dmax;               // one float, max of the dose
     double *host_err;          // pinned, 4 doubles: the optimiser's E and VER counts
     vamrt::OpParams op;
+    int ring_s;                // angles per group of the grouped operators; 0: not set up
+    float *ring_vols;          // 4 rotated copies of the volume
+    unsigned char *ring_bricks;
+    double2 *ring_cs;
+    int *ring_members;
+    CUtensorMap *ring_maps;
+    vamrt::RingParams ring;
 };
 
 namespace vamrt {
@@ -113,6 +138,14 @@ cudaError_t launch_forward_acc(const vamrt_projector *p, const void *proj, vamrt
                                cudaStream_t s);
 cudaError_t launch_unpad_acc(const vamrt_projector *p, const float *acc, void *dose, vamrt_dtype dt, uint32_t flags,
                              cudaStream_t s);
+
+// ring_project.cu: the projection over groups of angles.  Partition the angles (plan), tensor
+// maps of the rotated copies, and the launches: spread = caller's volume -> rotated copies.
+int plan_ring_groups(const double *theta, int n, int max_s, std::vector<int> &members, std::vector<double> &base);
+int ring_ex_classes(int S);
+cudaError_t ring_maps(const RingParams &G, int S, const float *vols, std::vector<CUtensorMap> &maps);
+cudaError_t launch_ring_spread(const vamrt_projector *p, const void *vol, vamrt_dtype dt, cudaStream_t s);
+cudaError_t launch_ring_project(const vamrt_projector *p, void *proj, vamrt_dtype dt, uint32_t flags, cudaStream_t s);
 
 // loss.cu: loss3 = device doubles {L, 1/|P|, 1/|Q|}; grad may be NULL
 cudaError_t launch_threshold_loss(const vamrt_projector *p, const void *dose, vamrt_dtype dose_dt,

@@ -156,6 +156,11 @@ void release(vamrt_projector *p)
     cudaFree(p->red);
     cudaFree(p->hist);
     cudaFree(p->dmax);
+    cudaFree(p->ring_vols);
+    cudaFree(p->ring_bricks);
+    cudaFree(p->ring_cs);
+    cudaFree(p->ring_members);
+    cudaFree(p->ring_maps);
     if (p->host_err) cudaFreeHost(p->host_err);
     if (cur >= 0 && cur != p->device) cudaSetDevice(cur);
     delete p;
@@ -165,6 +170,80 @@ struct Guard {
     vamrt_projector *p;
     ~Guard() { release(p); }
 };
+
+// The grouped operators' groups, rotated copies and tensor maps (ring.cu).  They need four
+// times the scratch volume; a handle that cannot have it, or whose grid is longer than the
+// kernels' window arithmetic and launch grids reach, keeps the per-angle operators.
+vamrt_status setup_ring(vamrt_projector *p, const std::vector<double> &theta, cudaStream_t s)
+{
+    const vamrt_geometry &g = p->g;
+    p->ring_s = 0;
+    if (g.nx > 8192 || g.ny > 8192 || g.nz > 8192) return VAMRT_OK;
+    vamrt::RingParams &G = p->ring;
+    G.op = p->op;
+    G.pzp = (g.nz + 2 + 3) & ~3;
+    G.vol_elems = (int64_t)(g.nx + 2) * (g.ny + 2) * G.pzp;
+    if (cudaMalloc(&p->ring_vols, sizeof(float) * 4 * (size_t)G.vol_elems) != cudaSuccess) {
+        cudaGetLastError();
+        p->ring_vols = nullptr;
+        return VAMRT_OK;
+    }
+    std::vector<int> members;
+    std::vector<double2> cs;
+    std::vector<CUtensorMap> maps;
+    int S = 0;
+    cudaError_t e = cudaSuccess;
+    try {
+        std::vector<double> base;
+        S = vamrt::plan_ring_groups(theta.data(), (int)theta.size(), g.nx == g.ny ? 4 : 2, members, base);
+        for (double th : base) cs.push_back(make_double2(cos(th), sin(th)));
+        e = vamrt::ring_maps(G, S, p->ring_vols, maps);
+    } catch (...) {
+        return fail(VAMRT_ENOMEM, "host allocation failed");
+    }
+    if (e == cudaErrorNotSupported) return VAMRT_OK;    // no tensor-map encoder
+    if (e != cudaSuccess) return cuda_fail(e, "tensor maps");
+    G.bzp = ((G.pzp + 7) / 8 + 7) & ~7;
+    G.brick_stride = (int64_t)((g.nx + 2 + 7) / 8) * ((g.ny + 2 + 7) / 8) * G.bzp;
+    CK(cudaMalloc(&p->ring_bricks, (size_t)(4 / S) * G.brick_stride), "cudaMalloc(bricks)");
+    CK(cudaMalloc(&p->ring_cs, sizeof(double2) * cs.size()), "cudaMalloc(groups)");
+    CK(cudaMalloc(&p->ring_members, sizeof(int) * members.size()), "cudaMalloc(groups)");
+    CK(cudaMalloc(&p->ring_maps, sizeof(CUtensorMap) * maps.size()), "cudaMalloc(tensor maps)");
+    CK(cudaMemcpyAsync(p->ring_cs, cs.data(), sizeof(double2) * cs.size(), cudaMemcpyHostToDevice, s), "copy");
+    CK(cudaMemcpyAsync(p->ring_members, members.data(), sizeof(int) * members.size(), cudaMemcpyHostToDevice, s), "copy");
+    CK(cudaMemcpyAsync(p->ring_maps, maps.data(), sizeof(CUtensorMap) * maps.size(), cudaMemcpyHostToDevice, s), "copy");
+    CK(cudaStreamSynchronize(s), "sync");
+    G.n_groups = (int)cs.size();
+    G.cs = p->ring_cs;
+    G.members = p->ring_members;
+    G.bricks = p->ring_bricks;
+    G.maps = p->ring_maps;
+    G.n_ex = vamrt::ring_ex_classes(S);
+    p->device_bytes += sizeof(float) * 4 * (uint64_t)G.vol_elems + (uint64_t)(4 / S) * G.brick_stride + (sizeof(double2) + sizeof(int) * S) * (uint64_t)cs.size() +
+                       sizeof(CUtensorMap) * (uint64_t)maps.size();
+    p->ring_s = S;
+    return VAMRT_OK;
+}
+
+// proj (+)= A^T vol
+cudaError_t project(const vamrt_projector *p, const void *vol, vamrt_dtype vol_dt, void *proj, vamrt_dtype proj_dt,
+                    uint32_t flags, cudaStream_t s)
+{
+    if (p->ring_s) {
+        const cudaError_t e = vamrt::launch_ring_spread(p, vol, vol_dt, s);
+        return e == cudaSuccess ? vamrt::launch_ring_project(p, proj, proj_dt, flags, s) : e;
+    }
+    const cudaError_t e = vamrt::launch_pad(p, vol, vol_dt, s);
+    return e == cudaSuccess ? vamrt::launch_adjoint(p, vol_dt, proj, proj_dt, flags, s) : e;
+}
+
+// dose (+)= A proj
+cudaError_t dose_to(const vamrt_projector *p, const void *proj, vamrt_dtype proj_dt, void *dose, vamrt_dtype dose_dt,
+                    uint32_t flags, cudaStream_t s)
+{
+    const cudaError_t e = vamrt::launch_forward(p, proj, proj_dt, s);
+    return e == cudaSuccess ? vamrt::launch_unpad(p, dose, dose_dt, flags, s) : e;
+}
 
 }  // namespace
 
@@ -237,16 +316,21 @@ vamrt_status vamrt_make_projector(const vamrt_geometry *geom, void *stream, vamr
     p->device_bytes = (sizeof(double4_32a) * 2 + sizeof(int2)) * (uint64_t)p->n_rays + sizeof(double2) * g.n_angles +
                       sizeof(float) * (uint64_t)p->pad_elems;
 
-    // angle table, FP64 on the host then rounded
-    double2 *hcs = (double2 *)malloc(sizeof(double2) * g.n_angles);
-    if (!hcs) return fail(VAMRT_ENOMEM, "host allocation failed");
-    for (int k = 0; k < g.n_angles; ++k) {
-        const double th = geom->angles_rad ? geom->angles_rad[k] : 2.0 * M_PI * k / g.n_angles;
-        hcs[k] = make_double2(cos(th), sin(th));
+    // angle table, FP64
+    std::vector<double> theta;
+    std::vector<double2> hcs;
+    try {
+        theta.resize((size_t)g.n_angles);
+        hcs.resize((size_t)g.n_angles);
+    } catch (...) {
+        return fail(VAMRT_ENOMEM, "host allocation failed");
     }
-    cudaError_t e = cudaMemcpyAsync(p->cs, hcs, sizeof(double2) * g.n_angles, cudaMemcpyHostToDevice, s);
+    for (int k = 0; k < g.n_angles; ++k) {
+        theta[(size_t)k] = geom->angles_rad ? geom->angles_rad[k] : 2.0 * M_PI * k / g.n_angles;
+        hcs[(size_t)k] = make_double2(cos(theta[(size_t)k]), sin(theta[(size_t)k]));
+    }
+    cudaError_t e = cudaMemcpyAsync(p->cs, hcs.data(), sizeof(double2) * g.n_angles, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    free(hcs);
     if (e != cudaSuccess) return cuda_fail(e, "angle table upload");
 
     // pupil samples, counters and the lens train (5 doubles per surface) in one temporary
@@ -314,6 +398,8 @@ vamrt_status vamrt_make_projector(const vamrt_geometry *geom, void *stream, vamr
     // a segment crosses the (-1,1)^3 neighbourhood of a voxel over at most 2 sqrt(3)
     // voxels; consecutive samples are more than step_vox / 2 apart (K = ceil(ell/ds))
     P.cell_bound = (float)fmax(2.0, floor(4.0 * sqrt(3.0) / g.step_vox) + 1.0);
+    st = setup_ring(p, theta, s);
+    if (st != VAMRT_OK) return st;
 
     guard.p = nullptr;
     *out = p;
@@ -347,8 +433,7 @@ vamrt_status vamrt_adjoint(vamrt_projector *p, const void *vol, vamrt_dtype vol_
     if (flags & ~(VAMRT_ACCUMULATE | VAMRT_CLAMP_NONNEG | VAMRT_UNATTENUATED))
         return fail(VAMRT_EINVAL, "unknown flags 0x%x", flags);
     cudaStream_t s = (cudaStream_t)stream;
-    CK(vamrt::launch_pad(p, vol, vol_dtype, s), "pad kernel");
-    CK(vamrt::launch_adjoint(p, vol_dtype, proj, proj_dtype, flags, s), "adjoint kernel");
+    CK(project(p, vol, vol_dtype, proj, proj_dtype, flags, s), "adjoint kernels");
     return VAMRT_OK;
 }
 
@@ -359,8 +444,7 @@ vamrt_status vamrt_forward_dose(vamrt_projector *p, const void *proj, vamrt_dtyp
     if (check_dtype(proj_dtype) || check_dtype(dose_dtype)) return VAMRT_EINVAL;
     if (flags & ~VAMRT_ACCUMULATE) return fail(VAMRT_EINVAL, "unknown flags 0x%x", flags);
     cudaStream_t s = (cudaStream_t)stream;
-    CK(vamrt::launch_forward(p, proj, proj_dtype, s), "forward kernel");
-    CK(vamrt::launch_unpad(p, dose, dose_dtype, flags, s), "unpad kernel");
+    CK(dose_to(p, proj, proj_dtype, dose, dose_dtype, flags, s), "forward kernels");
     return VAMRT_OK;
 }
 
@@ -419,8 +503,7 @@ vamrt_status optimize_gradient(vamrt_projector *p, const float *target, float *m
     if (params->timing) CK(cudaEventRecord(ev[0], s), "cudaEventRecord");
 
     // scale the start so that the part's mean dose is 1 (the thresholds' scale)
-    CK(vamrt::launch_forward(p, proj, pdt, s), "forward kernel");
-    CK(vamrt::launch_unpad(p, dose, ddt, 0u, s), "unpad kernel");
+    CK(dose_to(p, proj, pdt, dose, ddt, 0u, s), "forward kernels");
     CK(vamrt::launch_masked_sum(p, dose, ddt, target, nvox, sc2, s), "masked sum");
     double cnt[2];
     CK(cudaMemcpyAsync(cnt, sc2, sizeof(cnt), cudaMemcpyDeviceToHost, s), "copy");
@@ -450,16 +533,14 @@ vamrt_status optimize_gradient(vamrt_projector *p, const float *target, float *m
     for (; it < params->max_iter;) {
         if (params->timing) CK(cudaEventRecord(ev[0], s), "cudaEventRecord");
         // D = A g (stored in dose_dtype); L and dL/dD (FP32, in the model buffer)
-        CK(vamrt::launch_forward(p, proj, pdt, s), "forward kernel");
-        CK(vamrt::launch_unpad(p, dose, ddt, 0u, s), "unpad kernel");
+        CK(dose_to(p, proj, pdt, dose, ddt, 0u, s), "forward kernels");
         if (params->timing) CK(cudaEventRecord(ev[1], s), "cudaEventRecord");
         CK(vamrt::launch_threshold_loss(p, dose, ddt, target, (float)d_l, (float)d_h, loss3, model, VAMRT_F32, s),
            "threshold loss");
         CK(cudaMemcpyAsync(p->hist + it, loss3, sizeof(double), cudaMemcpyDeviceToDevice, s), "copy");
         if (params->timing) CK(cudaEventRecord(ev[2], s), "cudaEventRecord");
         // the projections' gradient A^T dL/dD
-        CK(vamrt::launch_pad(p, model, VAMRT_F32, s), "pad kernel");
-        CK(vamrt::launch_adjoint(p, VAMRT_F32, gradp, VAMRT_F32, 0u, s), "adjoint kernel");
+        CK(project(p, model, VAMRT_F32, gradp, VAMRT_F32, 0u, s), "adjoint kernels");
         if (params->timing) CK(cudaEventRecord(ev[3], s), "cudaEventRecord");
         // projected Adam step on the FP32 master (g >= 0), storage copy refreshed
         CK(vamrt::nn_adam(master, gradp, mom1, mom2, pdt == VAMRT_BF16 ? proj : nullptr, n, lr, 0.9f, 0.999f, 1e-12f,
@@ -562,12 +643,11 @@ vamrt_status vamrt_optimize(vamrt_projector *p, const float *target, float *mode
         if (params->timing) CK(cudaEventRecord(ev[0], s), "cudaEventRecord");
         if (!proj_space) {
             // g = max(0, A^T m)
-            CK(vamrt::launch_pad(p, model, VAMRT_F32, s), "pad kernel");
-            CK(vamrt::launch_adjoint(p, VAMRT_F32, proj, params->proj_dtype, VAMRT_CLAMP_NONNEG, s), "adjoint kernel");
+            CK(project(p, model, VAMRT_F32, proj, params->proj_dtype, VAMRT_CLAMP_NONNEG, s), "adjoint kernels");
         }
         if (params->timing) CK(cudaEventRecord(ev[1], s), "cudaEventRecord");
         // d = A g (left in the scratch volume), then normalise, update, error
-        CK(vamrt::launch_forward(p, proj, params->proj_dtype, s), "forward kernel");
+        CK(vamrt::launch_forward(p, proj, params->proj_dtype, s), "forward kernels");
         if (params->timing) CK(cudaEventRecord(ev[2], s), "cudaEventRecord");
         CK(vamrt::launch_osmo_step(p, target, model, dose, params->dose_dtype, fsum, p->hist + it, proj_space ? 1 : 0,
                                    (float)step, (float)params->momentum,
@@ -575,9 +655,8 @@ vamrt_status vamrt_optimize(vamrt_projector *p, const float *target, float *mode
            "osmo step");
         if (proj_space) {
             // g <- max(0, g + A^T (f - dn)); the residual is in the model buffer
-            CK(vamrt::launch_pad(p, model, VAMRT_F32, s), "pad kernel");
-            CK(vamrt::launch_adjoint(p, VAMRT_F32, proj, params->proj_dtype, VAMRT_ACCUMULATE | VAMRT_CLAMP_NONNEG, s),
-               "adjoint kernel");
+            CK(project(p, model, VAMRT_F32, proj, params->proj_dtype, VAMRT_ACCUMULATE | VAMRT_CLAMP_NONNEG, s),
+               "adjoint kernels");
         }
         if (params->timing) {
             CK(cudaEventRecord(ev[3], s), "cudaEventRecord");
