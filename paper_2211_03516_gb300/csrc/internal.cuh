@@ -60,6 +60,7 @@ struct RingParams {
     int64_t brick_stride;  // bricks of one copy
     const CUtensorMap *maps;   // device: [copy][EX class][EZ class]
     int n_ex;              // EX classes
+    float share_scale;     // fixed-point units of the largest ray weight (dose)
 };
 
 // Per-ray constants of the FP64 tracer.
@@ -101,8 +102,9 @@ struct vamrt_projector {
     float *dmax;               // one float, max of the dose
     double *host_err;          // pinned, 4 doubles: the optimiser's E and VER counts
     vamrt::OpParams op;
-    int ring_s;                // angles per group of the grouped operators; 0: not set up
-    float *ring_vols;          // 4 rotated copies of the volume
+    int ring_s;                // angles per group of the grouped projection; 0: not set up
+    int ring_dose;             // the dose is grouped too
+    float *ring_vols;          // 4 rotated copies of the volume, or dose accumulators
     unsigned char *ring_bricks;
     double2 *ring_cs;
     int *ring_members;
@@ -146,6 +148,12 @@ int ring_ex_classes(int S);
 cudaError_t ring_maps(const RingParams &G, int S, const float *vols, std::vector<CUtensorMap> &maps);
 cudaError_t launch_ring_spread(const vamrt_projector *p, const void *vol, vamrt_dtype dt, cudaStream_t s);
 cudaError_t launch_ring_project(const vamrt_projector *p, void *proj, vamrt_dtype dt, uint32_t flags, cudaStream_t s);
+
+// ring_dose.cu: the dose over groups of angles into four rotated accumulators, and their sum
+// -> out at the given pitches (elements).
+cudaError_t launch_ring_dose(const vamrt_projector *p, const void *proj, vamrt_dtype dt, cudaStream_t s);
+cudaError_t launch_ring_gather(const vamrt_projector *p, void *out, vamrt_dtype dt, int64_t row, int64_t plane,
+                               int64_t origin, int accumulate, cudaStream_t s);
 
 // loss.cu: loss3 = device doubles {L, 1/|P|, 1/|Q|}; grad may be NULL
 cudaError_t launch_threshold_loss(const vamrt_projector *p, const void *dose, vamrt_dtype dose_dt,

@@ -5,10 +5,9 @@
 // theta + 180 degrees (N even) and theta + 90, 270 (N a multiple of 4, square grids).  A
 // quarter turn maps the voxel lattice onto itself, so ray r at theta + 90 i samples the
 // volume turned back by 90 i degrees at exactly the positions it samples the volume itself
-// at theta.  All S angles of such a group (S = 4 or 2; S = 1 when the scan has no partners)
-// are walked at once: one ray set-up in FP64, one position, one cell and one set of
+// at theta.  All S angles of such a group (S = 4 or 2) are walked at once: one ray set-up in FP64, one position, one cell and one set of
 // trilinear weights per sample serve S angles.  The projection reads the S rotated volumes
-// interleaved, one 16-byte (8, 4) shared-memory read per corner; the dose adds into S
+// interleaved, one 16-byte (8) shared-memory read per corner; the dose (S = 4 only) adds into
 // rotated accumulators.  Positions are those of the group's first angle: cos and sin of
 // the partners would differ from its turned ones by FP64 rounding only (1e-16 rad).
 //
@@ -140,8 +139,9 @@ __device__ __forceinline__ void slot_reset(int *s, int k)
 __device__ __forceinline__ int fix8(long long q) { return (int)(q >> 24); }   // Q32.32 -> 1/256 voxel, floored
 
 // Block-uniform; every thread calls it with its ray (placed rays when it returns).  `align`:
-// z alignment of the window's corner; `exq`: EX granularity.  Returns false when the block has no active ray.
-__device__ __forceinline__ bool bundle(const RingParams &G, int *s, bool active, RRay &R, int align,
+// z alignment of the window's corner; `exq`: EX granularity; bad_ray:
+// the ray wants the walk on global memory.  Returns false when the block has no active ray.
+__device__ __forceinline__ bool bundle(const RingParams &G, int *s, bool active, bool bad_ray, RRay &R, int align,
                                        int exq, int cap, bool split, int &turn, Window &W)
 {
     const bool lead = threadIdx.x == 0;
@@ -161,7 +161,7 @@ __device__ __forceinline__ bool bundle(const RingParams &G, int *s, bool active,
     if (active) {
         place(G, turn, R);
         const long long m = max(llabs(R.sx), llabs(R.sz));
-        bad = 4 * R.sy >= m && R.sy > 0 ? 0 : 1;
+        bad = 4 * R.sy >= m && R.sy > 0 && !bad_ray ? 0 : 1;
         const int yf = (int)(R.qy >> 32), yl = (int)((R.qy + (long long)(R.jhi - 1 - R.j) * R.sy) >> 32);
         ylo = min(yf, yl);
         yhi = max(yf, yl) + 1;
@@ -292,14 +292,15 @@ __device__ __forceinline__ int samples_below(const RRay &R, int lim)
 }
 
 // Walks the ray's samples with row < lim, at most n of them: flush(e, y, run) is called
-// once per run of samples in one cell, at x zpitch + z = e of row y.
+// once per run of samples in one cell, at x zpitch + z = e of row y.  Weights carry `unit`
+// (a power of two).
 template <typename F>
-__device__ __forceinline__ void walk(RRay &R, float ratio, int n, int lim, int zpitch, F &&flush)
+__device__ __forceinline__ void walk(RRay &R, float ratio, float unit, int n, int lim, int zpitch, F &&flush)
 {
     int y = (int)(R.qy >> 32);
     n = min(n, R.jhi - R.j);
     if (n <= 0 || y >= lim) return;
-    float att = exp2f(R.att * ((float)R.j + 0.5f));      // exact at each stage, then one product per sample
+    float att = unit * exp2f(R.att * ((float)R.j + 0.5f));   // exact at each stage, then one product per sample
     const int last = R.j + n;
     Run r;
     r.clear();
@@ -325,9 +326,9 @@ __device__ __forceinline__ void walk(RRay &R, float ratio, int n, int lim, int z
 
 // component of angle i of a group when the block's turn is r, and the volume it lies in
 template <int S>
-__device__ __forceinline__ int volume_of(int r) { return S == 4 ? 0 : S == 2 ? (r & 1) : r; }
+__device__ __forceinline__ int volume_of(int r) { return S == 4 ? 0 : (r & 1); }
 template <int S>
-__device__ __forceinline__ int shift_of(int r) { return S == 4 ? r : S == 2 ? (r >> 1) : 0; }
+__device__ __forceinline__ int shift_of(int r) { return S == 4 ? r : (r >> 1); }
 
 inline dim3 ring_grid(const RingParams &G, int columns)
 {
@@ -345,9 +346,7 @@ cudaError_t by_storage(vamrt_dtype dt, void *ptr, F &&f)
 template <typename F>
 cudaError_t by_group(int S, F &&f)
 {
-    if (S == 4) return f(std::integral_constant<int, 4>());
-    if (S == 2) return f(std::integral_constant<int, 2>());
-    return f(std::integral_constant<int, 1>());
+    return S == 4 ? f(std::integral_constant<int, 4>()) : f(std::integral_constant<int, 2>());
 }
 
 }  // namespace

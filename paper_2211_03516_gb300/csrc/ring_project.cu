@@ -32,7 +32,7 @@ namespace {
 constexpr int kProjTU = 8, kProjThreads = kProjTU * kRingTV;
 
 // Blocks per SM and ring words.  Four components (113 registers) take two blocks with 104 KB
-// each, longer stages; the others three with 68 KB (64^3, S = 2: 83 us against 94).
+// each, longer stages; two components three with 68 KB (64^3, 90 angles: 83 us against 94).
 template <int S>
 constexpr int kProjBlocks = S == 4 ? 2 : 3;
 template <int S>
@@ -75,7 +75,7 @@ __global__ void __launch_bounds__(256) spread_kernel(const VT *__restrict__ vol,
     if (t < kTileX / kBrick) lit[t] = 0;
 #pragma unroll
     for (int c = 0; c < S; ++c) {
-        const int r = S == 4 ? c : S == 2 ? 2 * c + w : w;
+        const int r = S == 4 ? c : 2 * c + w;
 #pragma unroll 4
         for (int i = t; i < kTileX * kTileY * kTileZ; i += 256) {
             const int zz = i >> 8, k = i & 255;
@@ -105,10 +105,8 @@ __global__ void __launch_bounds__(256) spread_kernel(const VT *__restrict__ vol,
         if (S == 4)
             *reinterpret_cast<float4 *>(p) =
                 make_float4(tile[0][zz][yy][xx], tile[1 % S][zz][yy][xx], tile[2 % S][zz][yy][xx], tile[3 % S][zz][yy][xx]);
-        else if (S == 2)
-            *reinterpret_cast<float2 *>(p) = make_float2(tile[0][zz][yy][xx], tile[1 % S][zz][yy][xx]);
         else
-            *p = tile[0][zz][yy][xx];
+            *reinterpret_cast<float2 *>(p) = make_float2(tile[0][zz][yy][xx], tile[1][zz][yy][xx]);
     }
     if (__any_sync(kFull, any) && (t & 31) == 0) lit[t >> 6] = 1;      // two warps store the same value
     __syncthreads();
@@ -150,10 +148,8 @@ __device__ __forceinline__ void ld_shared(float (&v)[S], uint32_t p)
 {
     if constexpr (S == 4)
         asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]) : "r"(p));
-    else if constexpr (S == 2)
-        asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v[0]), "=f"(v[1]) : "r"(p));
     else
-        asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v[0]) : "r"(p));
+        asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v[0]), "=f"(v[1]) : "r"(p));
 }
 template <int S>
 __device__ __forceinline__ void ld_global(float (&v)[S], const float *p)
@@ -161,11 +157,9 @@ __device__ __forceinline__ void ld_global(float (&v)[S], const float *p)
     if constexpr (S == 4) {
         const float4 q = __ldg(reinterpret_cast<const float4 *>(p));
         v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
-    } else if constexpr (S == 2) {
+    } else {
         const float2 q = __ldg(reinterpret_cast<const float2 *>(p));
         v[0] = q.x; v[1] = q.y;
-    } else {
-        v[0] = __ldg(p);
     }
 }
 
@@ -257,7 +251,7 @@ __global__ void __launch_bounds__(kProjThreads, kProjBlocks<S>)
                             ring_ray(G, ((int64_t)(a % P.M) * P.nv + v) * P.nu + u, scs, R, flags & VAMRT_UNATTENUATED);
         if (!active) R.jhi = R.j = 0;
         Window W;
-        const bool any = bundle(G, slots[a % 3], active, R, kAlign, kExq, kProjWords<S> / S, true, turn, W);
+        const bool any = bundle(G, slots[a % 3], active, false, R, kAlign, kExq, kProjWords<S> / S, true, turn, W);
         if (tid < kSlots) slot_reset(slots[(a + 2) % 3], tid);      // last read one aperture sample ago
         if (tid == 0) sW = W;
         __syncthreads();
@@ -338,7 +332,7 @@ __global__ void __launch_bounds__(kProjThreads, kProjBlocks<S>)
             }
             float o[S] = {};
             const int ya = sW.y0 + cur * sW.R;
-            walk(R, ratio, INT_MAX, ya + sW.R, zpitch, [&](int e, int y, const Run &r) {
+            walk(R, ratio, 1.0f, INT_MAX, ya + sW.R, zpitch, [&](int e, int y, const Run &r) {
                 const int2 off = rowoff[b][y - ya];
                 const uint32_t at = ring0 + (uint32_t)(e * S * 4);
                 gather_shared<S>(o, r, at + off.x, at + off.y, zpitch * S * 4);
@@ -364,7 +358,7 @@ __global__ void __launch_bounds__(kProjThreads, kProjBlocks<S>)
             const int64_t row = (int64_t)(((turn & 1) ? P.ny : P.nx) + 2) * G.pzp;
             while (R.j < R.jhi) {
                 float o[S] = {};
-                walk(R, ratio, 16, INT_MAX, G.pzp, [&](int e, int y, const Run &r) {
+                walk(R, ratio, 1.0f, 16, INT_MAX, G.pzp, [&](int e, int y, const Run &r) {
                     const float *p = vol + (y * row + e) * S;
                     gather_global<S>(o, r, p, p + row * S, (int64_t)G.pzp * S);
                 });
@@ -393,11 +387,11 @@ __global__ void __launch_bounds__(kProjThreads, kProjBlocks<S>)
 
 }  // namespace
 
-// Partition angles into groups theta0 + i 2 pi / S, S the largest of `max_s`, 2, 1 for which
-// every angle has its partners (to 1e-12 rad).  members: S angle indices per group.
+// Partition angles into groups theta0 + i 2 pi / S, S the largest of `max_s` and 2 for which every
+// angle has its partners (to 1e-12 rad); 0 without partners.  members: S angle indices per group.
 int plan_ring_groups(const double *theta, int n, int max_s, std::vector<int> &members, std::vector<double> &base)
 {
-    for (int S = max_s; S >= 1; S >>= 1) {
+    for (int S = max_s; S >= 2; S >>= 1) {
         const double turn = 2.0 * M_PI / S;
         if (n % S) continue;
         struct Item {
@@ -427,7 +421,7 @@ int plan_ring_groups(const double *theta, int n, int max_s, std::vector<int> &me
         }
         if (good) return S;
     }
-    return 0;   // not reached: S = 1 always groups
+    return 0;
 }
 
 int ring_ex_classes(int S) { return (kMaxEX - kMinEX) / (4 / S) + 1; }

@@ -171,37 +171,59 @@ struct Guard {
     ~Guard() { release(p); }
 };
 
-// The grouped operators' groups, rotated copies and tensor maps (ring.cu).  They need four
-// times the scratch volume; a handle that cannot have it, or whose grid is longer than the
-// kernels' window arithmetic and launch grids reach, keeps the per-angle operators.
+// Whether a scan of `blocks` pixel tiles x angles is large enough for the grouped operators, whose
+// blocks do S angles' work each.  The per-angle kernels hold 3 blocks per SM.
+//   Projection: worth it once those take more than one wave (64^3, 12 angles, 192 blocks:
+//   grouped 40 us, per angle 37; 36 angles, 576 blocks: 41 against 61).
+//   Dose: more than three (54 x 54 x 76, 4 rays, 48 angles, 1296 blocks: 264 against 212 us;
+//   128^3, 24 angles, 1536 blocks: 643 against 716).
+bool grouped_projection_pays(const vamrt_projector *p, int64_t blocks) { return blocks > 3 * (int64_t)p->num_sms; }
+bool grouped_dose_pays(const vamrt_projector *p, int64_t blocks) { return blocks > 9 * (int64_t)p->num_sms; }
+
+// The grouped operators' groups, rotated copies and tensor maps (ring.cuh).  Scans without
+// partner angles, small scans, handles that cannot have four times the scratch volume, and
+// grids longer than the kernels' window arithmetic and launch grids reach keep the per-angle
+// operators.
 vamrt_status setup_ring(vamrt_projector *p, const std::vector<double> &theta, cudaStream_t s)
 {
     const vamrt_geometry &g = p->g;
     p->ring_s = 0;
-    if (g.nx > 8192 || g.ny > 8192 || g.nz > 8192) return VAMRT_OK;
+    p->ring_dose = 0;
+    const int64_t blocks = (int64_t)((g.nu + 7) / 8) * ((g.nv + 31) / 32) * g.n_angles;
+    if (!grouped_projection_pays(p, blocks) || g.nx > 8192 || g.ny > 8192 || g.nz > 8192) return VAMRT_OK;
     vamrt::RingParams &G = p->ring;
     G.op = p->op;
     G.pzp = (g.nz + 2 + 3) & ~3;
     G.vol_elems = (int64_t)(g.nx + 2) * (g.ny + 2) * G.pzp;
+    if (G.vol_elems >= (int64_t)1 << 31) return VAMRT_OK;
+    std::vector<int> members;
+    std::vector<double2> cs;
+    std::vector<CUtensorMap> maps;
+    int S = 0;
+    try {
+        std::vector<double> base;
+        S = vamrt::plan_ring_groups(theta.data(), (int)theta.size(), g.nx == g.ny ? 4 : 2, members, base);
+        for (double th : base) cs.push_back(make_double2(cos(th), sin(th)));
+    } catch (...) {
+        return fail(VAMRT_ENOMEM, "host allocation failed");
+    }
+    if (S == 0) return VAMRT_OK;                        // no partners
     if (cudaMalloc(&p->ring_vols, sizeof(float) * 4 * (size_t)G.vol_elems) != cudaSuccess) {
         cudaGetLastError();
         p->ring_vols = nullptr;
         return VAMRT_OK;
     }
-    std::vector<int> members;
-    std::vector<double2> cs;
-    std::vector<CUtensorMap> maps;
-    int S = 0;
     cudaError_t e = cudaSuccess;
     try {
-        std::vector<double> base;
-        S = vamrt::plan_ring_groups(theta.data(), (int)theta.size(), g.nx == g.ny ? 4 : 2, members, base);
-        for (double th : base) cs.push_back(make_double2(cos(th), sin(th)));
         e = vamrt::ring_maps(G, S, p->ring_vols, maps);
     } catch (...) {
         return fail(VAMRT_ENOMEM, "host allocation failed");
     }
-    if (e == cudaErrorNotSupported) return VAMRT_OK;    // no tensor-map encoder
+    if (e == cudaErrorNotSupported) {                   // no tensor-map encoder
+        cudaFree(p->ring_vols);
+        p->ring_vols = nullptr;
+        return VAMRT_OK;
+    }
     if (e != cudaSuccess) return cuda_fail(e, "tensor maps");
     G.bzp = ((G.pzp + 7) / 8 + 7) & ~7;
     G.brick_stride = (int64_t)((g.nx + 2 + 7) / 8) * ((g.ny + 2 + 7) / 8) * G.bzp;
@@ -219,9 +241,15 @@ vamrt_status setup_ring(vamrt_projector *p, const std::vector<double> &theta, cu
     G.bricks = p->ring_bricks;
     G.maps = p->ring_maps;
     G.n_ex = vamrt::ring_ex_classes(S);
+    // Fixed-point units of the largest weight: a voxel's sum over a block's 256 rays stays
+    // below 2^31, and one share -- up to the floor(2 sqrt(3) / step) + 1 samples of a ray in
+    // one cell -- below the 2^22 that its conversion holds.
+    const double run = floor(2.0 * sqrt(3.0) / g.step_vox) + 1.0;
+    G.share_scale = (float)fmin(2147483648.0 / (1.01 * 256.0 * p->op.cell_bound), 4.1e6 / run);
     p->device_bytes += sizeof(float) * 4 * (uint64_t)G.vol_elems + (uint64_t)(4 / S) * G.brick_stride + (sizeof(double2) + sizeof(int) * S) * (uint64_t)cs.size() +
                        sizeof(CUtensorMap) * (uint64_t)maps.size();
     p->ring_s = S;
+    p->ring_dose = S == 4 && grouped_dose_pays(p, blocks) ? 1 : 0;
     return VAMRT_OK;
 }
 
@@ -241,8 +269,24 @@ cudaError_t project(const vamrt_projector *p, const void *vol, vamrt_dtype vol_d
 cudaError_t dose_to(const vamrt_projector *p, const void *proj, vamrt_dtype proj_dt, void *dose, vamrt_dtype dose_dt,
                     uint32_t flags, cudaStream_t s)
 {
+    if (p->ring_dose) {
+        const cudaError_t e = vamrt::launch_ring_dose(p, proj, proj_dt, s);
+        const int64_t nx = p->g.nx, ny = p->g.ny;
+        return e == cudaSuccess ? vamrt::launch_ring_gather(p, dose, dose_dt, nx, nx * ny, 0,
+                                                            (flags & VAMRT_ACCUMULATE) ? 1 : 0, s)
+                                : e;
+    }
     const cudaError_t e = vamrt::launch_forward(p, proj, proj_dt, s);
     return e == cudaSuccess ? vamrt::launch_unpad(p, dose, dose_dt, flags, s) : e;
+}
+
+// the FP32 dose A proj in the padded scratch volume (its halo is undefined)
+cudaError_t dose_in_scratch(const vamrt_projector *p, const void *proj, vamrt_dtype proj_dt, cudaStream_t s)
+{
+    if (!p->ring_dose) return vamrt::launch_forward(p, proj, proj_dt, s);
+    const cudaError_t e = vamrt::launch_ring_dose(p, proj, proj_dt, s);
+    const int64_t row = p->op.px, plane = row * p->op.py;
+    return e == cudaSuccess ? vamrt::launch_ring_gather(p, p->scratch, VAMRT_F32, row, plane, plane + row + 1, 0, s) : e;
 }
 
 }  // namespace
@@ -647,7 +691,7 @@ vamrt_status vamrt_optimize(vamrt_projector *p, const float *target, float *mode
         }
         if (params->timing) CK(cudaEventRecord(ev[1], s), "cudaEventRecord");
         // d = A g (left in the scratch volume), then normalise, update, error
-        CK(vamrt::launch_forward(p, proj, params->proj_dtype, s), "forward kernels");
+        CK(dose_in_scratch(p, proj, params->proj_dtype, s), "forward kernels");
         if (params->timing) CK(cudaEventRecord(ev[2], s), "cudaEventRecord");
         CK(vamrt::launch_osmo_step(p, target, model, dose, params->dose_dtype, fsum, p->hist + it, proj_space ? 1 : 0,
                                    (float)step, (float)params->momentum,

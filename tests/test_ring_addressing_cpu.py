@@ -17,7 +17,7 @@ from oracle import vam_oracle as O
 from paper_2211_03516_gb300 import inputs as I
 
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2211_03516_gb300", "csrc")
-SRC = "".join(open(os.path.join(CSRC, f)).read() for f in ("ring.cuh", "ring_project.cu"))
+SRC = "".join(open(os.path.join(CSRC, f)).read() for f in ("ring.cuh", "ring_project.cu", "ring_dose.cu"))
 f32 = np.float32
 
 
@@ -30,8 +30,11 @@ def const(name):
 TU, TV = const("kProjTU"), const("kRingTV")
 MAX_EX, MAX_EZ, MIN_EX, STEP_EZ, TAB = (const(n) for n in ("kMaxEX", "kMaxEZ", "kMinEX", "kStepEZ", "kRowTab"))
 WORDS = [int(eval(x)) for x in re.search(r"kProjWords = S == 4 \? ([0-9 *]+) : ([0-9 *]+);", SRC).groups()]
-# (alignment of z, granularity of EX, voxels of the ring, two buffers): projection, 4, 2 and 1 angles
-FORMS = [(4 // S, 4 // S, WORDS[S != 4] // S, True) for S in (4, 2, 1)]
+DOSE_WORDS = const("kDoseWords")
+# (alignment of z, granularity of EX, voxels of the ring, two buffers): projection of 4 and 2
+# angles, dose of 4
+FORMS = [(4 // S, 4 // S, WORDS[S != 4] // S, True) for S in (4, 2)] + [(4, 1, DOSE_WORDS // 4, False)]
+assert const("kDoseTU") == TU and 3 * ((TAB - 3) // 2) + 1 < const("kDoseTab")
 
 
 def q32(x):
