@@ -97,6 +97,7 @@ struct vamrt_projector {
     double2 *cs;
     float *scratch;            // padded FP32 volume, pad_elems floats
     int64_t pad_elems;
+    unsigned char *pad_bricks; // which 8^3 bricks of the padded volume hold anything
     double *red;               // kRedBlocks partials + scalars
     double *hist;              // kMaxHistory errors
     float *dmax;               // one float, max of the dose

@@ -51,6 +51,7 @@ namespace vamrt {
 namespace {
 
 constexpr double kFix = 4294967296.0;  // 2^32
+constexpr int kBrick = 8;
 constexpr unsigned kFull = 0xffffffffu;
 
 __device__ __forceinline__ float to_f(float x) { return x; }
@@ -94,20 +95,44 @@ __device__ __forceinline__ void red_v4(float *p, float4 v)
 // ---------------------------------------------------------------------------------
 // halo copy: scratch[zp][yp][xp] = vol[zp-1][yp-1][xp-1] inside, 0 elsewhere
 // ---------------------------------------------------------------------------------
+// A block takes 32 x by 8 y by 8 z padded voxels, a row per warp and plane; it also notes, per
+// 8^3 brick, whether any voxel is nonzero: bricks[z / 8][y / 8][x / 8].
+constexpr int kPadX = 32, kPadY = 8, kPadZ = 8;
 template <typename VT>
-__global__ void pad_kernel(const VT *__restrict__ vol, VT *__restrict__ out, int nx, int ny, int nz, int px,
-                           int py, int64_t total)
+__global__ void __launch_bounds__(kPadX *kPadY)
+    pad_kernel(const VT *__restrict__ vol, VT *__restrict__ out, unsigned char *__restrict__ bricks, int nx, int ny, int nz,
+               int px, int py, int pz)
 {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const int xp = (int)(i % px);
-        const int yp = (int)((i / px) % py);
-        const int zp = (int)(i / ((int64_t)px * py));
-        VT val = VT(0.0f);
-        if (xp >= 1 && xp <= nx && yp >= 1 && yp <= ny && zp >= 1 && zp <= nz)
-            val = vol[((int64_t)(zp - 1) * ny + (yp - 1)) * nx + (xp - 1)];
-        out[i] = val;
+    __shared__ int lit[kPadX / kBrick];
+    const int gx = (px + kPadX - 1) / kPadX, gy = (py + kPadY - 1) / kPadY;
+    const int tx = blockIdx.x % gx, zy = blockIdx.x / gx, ty = zy % gy, tz = zy / gy;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int x = tx * kPadX + lane, y = ty * kPadY + w, z0 = tz * kPadZ;
+    if (threadIdx.x < kPadX / kBrick) lit[threadIdx.x] = 0;
+    __syncthreads();
+    bool any = false;
+    if (x < px && y < py) {
+        const bool row = x >= 1 && x <= nx && y >= 1 && y <= ny;
+        VT val[kPadZ];
+#pragma unroll
+        for (int k = 0; k < kPadZ; ++k) {
+            const int z = z0 + k;
+            val[k] = VT(0.0f);
+            if (row && z >= 1 && z <= nz) val[k] = vol[((int64_t)(z - 1) * ny + (y - 1)) * nx + (x - 1)];
+        }
+#pragma unroll
+        for (int k = 0; k < kPadZ; ++k)
+            if (z0 + k < pz) {
+                out[((int64_t)(z0 + k) * py + y) * px + x] = val[k];
+                any |= to_f(val[k]) != 0.f;
+            }
     }
+    const unsigned m = __ballot_sync(kFull, any);
+    if (lane < kPadX / kBrick && (m >> (kBrick * lane) & 0xffu)) lit[lane] = 1;      // any warp stores the same value
+    __syncthreads();
+    const int bx = tx * (kPadX / kBrick) + threadIdx.x, nbx = (px + kBrick - 1) / kBrick;
+    if (threadIdx.x < kPadX / kBrick && bx < nbx)
+        bricks[((int64_t)tz * gy + ty) * nbx + bx] = (unsigned char)lit[threadIdx.x];
 }
 
 // dose[z][y][x] (+)= scratch[z+1][y+1][x+1]
@@ -535,8 +560,8 @@ constexpr int kMaxBoxExtent = 255;
 
 template <bool FWD, typename VT, typename PT>
 __global__ void __launch_bounds__(kThreads, kBlocksPerSm)
-    tiled_kernel(const OpParams P, const VT *__restrict__ vol, PT *__restrict__ proj, float *__restrict__ acc,
-                 uint32_t flags)
+    tiled_kernel(const OpParams P, const VT *__restrict__ vol, const unsigned char *__restrict__ bricks,
+                 PT *__restrict__ proj, float *__restrict__ acc, uint32_t flags)
 {
     extern __shared__ __align__(16) float box[];
     __shared__ int s_box[3][6];   // per chunk (rotating): min x,y,z and max x,y,z of the footprint
@@ -563,6 +588,7 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSm)
     const int pxy = P.px * P.py;
     float pix = 0.f;
     int n_chunk = 0;
+    int lit_run = 0;             // looks at the bricks since one found nothing
     for (int a = 0; a < P.M; ++a) {
         const int ra = a % 3;
         Ray R;
@@ -658,6 +684,25 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSm)
                 continue;
             }
             if (fits && in_grid) {
+                // A box that touches only empty bricks adds exactly nothing.  A look costs a barrier and
+                // a read per thread, so where four in a row have found something only every fourth
+                // box is looked at.  128^3, 45 angles: a part 1402 -> 986 us, a volume without a zero
+                // 1400 -> 1412 (1426 with a look at every box).
+                if (!FWD && (lit_run < 4 || (n_chunk & 3) == 0)) {
+                    const int kx = bx0 / kBrick, ky = by0 / kBrick, kz = bz0 / kBrick;
+                    const int cx = hx / kBrick - kx + 1, cy = hy / kBrick - ky + 1, cz = hz / kBrick - kz + 1;
+                    const int nbx = (P.px + kBrick - 1) / kBrick, nby = (P.py + kBrick - 1) / kBrick;
+                    int any = 0;
+                    for (int i = tid; i < cx * cy * cz; i += kThreads) {
+                        const int zy = fdiv(i, 1.0f / (float)cx), z = fdiv(zy, 1.0f / (float)cy);
+                        any |= __ldg(bricks + ((int64_t)(kz + z) * nby + (ky + zy - z * cy)) * nbx + (kx + i - zy * cx));
+                    }
+                    if (!__syncthreads_or(any)) {
+                        lit_run = 0;
+                        continue;
+                    }
+                    ++lit_run;
+                }
                 const SlotWalk sw(ex4, ey);
                 if (!FWD) {
                     const int64_t gstep = (int64_t)sw.phases * pxy;
@@ -749,12 +794,13 @@ inline dim3 op_grid(const OpParams &P)
 constexpr size_t kSmem = sizeof(float) * kBoxFloats;
 
 template <bool FWD, typename VT, typename PT>
-cudaError_t launch_tiled(const OpParams &P, const VT *vol, PT *proj, float *acc, uint32_t flags, cudaStream_t s)
+cudaError_t launch_tiled(const OpParams &P, const VT *vol, const unsigned char *bricks, PT *proj, float *acc,
+                         uint32_t flags, cudaStream_t s)
 {
     cudaError_t e = cudaFuncSetAttribute(tiled_kernel<FWD, VT, PT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)kSmem);
     if (e != cudaSuccess) return e;
-    tiled_kernel<FWD, VT, PT><<<op_grid(P), dim3(kTileV, kTileU), kSmem, s>>>(P, vol, proj, acc, flags);
+    tiled_kernel<FWD, VT, PT><<<op_grid(P), dim3(kTileV, kTileU), kSmem, s>>>(P, vol, bricks, proj, acc, flags);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -773,10 +819,12 @@ cudaError_t with_storage(vamrt_dtype dt, void *ptr, F &&f)
 cudaError_t launch_pad(const vamrt_projector *p, const void *vol, vamrt_dtype dt, cudaStream_t s)
 {
     const OpParams &P = p->op;
-    const unsigned grid = grid_for(p, p->pad_elems, 256);
+    // at most 2^31 / 2048 blocks
+    const unsigned grid = (unsigned)((P.px + kPadX - 1) / kPadX) * ((P.py + kPadY - 1) / kPadY) * ((P.pz + kPadZ - 1) / kPadZ);
     return with_storage(dt, const_cast<void *>(vol), [&](auto *v) {
         using VT = std::remove_pointer_t<decltype(v)>;
-        pad_kernel<VT><<<grid, 256, 0, s>>>(v, (VT *)p->scratch, P.nx, P.ny, P.nz, P.px, P.py, p->pad_elems);
+        pad_kernel<VT><<<grid, kPadX * kPadY, 0, s>>>(v, (VT *)p->scratch, p->pad_bricks, P.nx, P.ny, P.nz, P.px, P.py,
+                                                      P.pz);
         count_launches(1);
         return cudaGetLastError();
     });
@@ -788,7 +836,8 @@ cudaError_t launch_adjoint(const vamrt_projector *p, vamrt_dtype vol_dt, void *p
     const OpParams &P = p->op;
     return with_storage(vol_dt, p->scratch, [&](auto *vol) {
         return with_storage(proj_dt, proj, [&](auto *pr) {
-            return launch_tiled<false>(P, (const std::remove_pointer_t<decltype(vol)> *)vol, pr, nullptr, flags, s);
+            return launch_tiled<false>(P, (const std::remove_pointer_t<decltype(vol)> *)vol, p->pad_bricks, pr, nullptr, flags,
+                                       s);
         });
     });
 }
@@ -799,7 +848,7 @@ cudaError_t launch_forward_acc(const vamrt_projector *p, const void *proj, vamrt
     const OpParams &P = p->op;
     const float *none = nullptr;
     return with_storage(proj_dt, const_cast<void *>(proj),
-                        [&](auto *pr) { return launch_tiled<true>(P, none, pr, acc, 0u, s); });
+                        [&](auto *pr) { return launch_tiled<true>(P, none, nullptr, pr, acc, 0u, s); });
 }
 
 cudaError_t launch_forward(const vamrt_projector *p, const void *proj, vamrt_dtype proj_dt, cudaStream_t s)

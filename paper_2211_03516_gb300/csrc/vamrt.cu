@@ -153,6 +153,7 @@ void release(vamrt_projector *p)
     cudaFree(p->tabJ);
     cudaFree(p->cs);
     cudaFree(p->scratch);
+    cudaFree(p->pad_bricks);
     cudaFree(p->red);
     cudaFree(p->hist);
     cudaFree(p->dmax);
@@ -353,6 +354,8 @@ vamrt_status vamrt_make_projector(const vamrt_geometry *geom, void *stream, vamr
     CK(cudaMalloc(&p->tabJ, sizeof(int2) * p->n_rays), "cudaMalloc(ray table)");
     CK(cudaMalloc(&p->cs, sizeof(double2) * g.n_angles), "cudaMalloc(angles)");
     CK(cudaMalloc(&p->scratch, sizeof(float) * p->pad_elems), "cudaMalloc(scratch volume)");
+    const int64_t bricks = (int64_t)((px + 7) / 8) * ((g.ny + 2 + 7) / 8) * ((g.nz + 2 + 7) / 8);
+    CK(cudaMalloc(&p->pad_bricks, (size_t)bricks), "cudaMalloc(bricks)");
     CK(cudaMalloc(&p->red, sizeof(double) * (vamrt::kRedBlocks + 8)), "cudaMalloc(reduction)");
     CK(cudaMalloc(&p->hist, sizeof(double) * vamrt::kMaxHistory), "cudaMalloc(history)");
     CK(cudaMalloc(&p->dmax, sizeof(float) * 4), "cudaMalloc(dmax)");
