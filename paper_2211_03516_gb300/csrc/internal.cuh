@@ -46,6 +46,15 @@ struct OpParams {
     float h_over_m;       // voxel pitch (mm) / rays per pixel: delta_mm / M = delta_vox * h_over_m
 };
 
+// The voxel error rate's device state, cleared before each use: histograms of the in-part and
+// the out-of-part resin voxels, the dose's maximum over the resin, and blocks done.
+constexpr int kVerBins = 1024;
+struct VerState {
+    unsigned hist[2 * kVerBins];
+    float dmax;
+    unsigned counter;
+};
+
 // Per-launch constants of the grouped operators (ring.cuh).  Groups of S angles a quarter,
 // half or whole turn apart are walked together on rotated copies of the volume.
 struct RingParams {
@@ -100,7 +109,8 @@ struct vamrt_projector {
     unsigned char *pad_bricks; // which 8^3 bricks of the padded volume hold anything
     double *red;               // kRedBlocks partials + scalars
     double *hist;              // kMaxHistory errors
-    float *dmax;               // one float, max of the dose
+    vamrt::VerState *ver;
+    int2 *spans;               // per y: [first, end) resin voxel of the row
     double *host_err;          // pinned, 4 doubles: the optimiser's E and VER counts
     vamrt::OpParams op;
     int ring_s;                // angles per group of the grouped projection; 0: not set up
@@ -169,7 +179,9 @@ cudaError_t launch_masked_sum(const vamrt_projector *p, const void *x, vamrt_dty
 cudaError_t launch_scale_master(const vamrt_projector *p, void *x, vamrt_dtype dt, float *master, int64_t n, float sc,
                                 cudaStream_t s);
 
-// ver.cu: out3 = device {best mismatch count, best threshold index, resin voxels}
+// ver.cu: the resin rows' ends (once per handle); out3 = device {best mismatch count, best
+// threshold index, resin voxels}
+cudaError_t launch_resin_spans(const vamrt_projector *p, cudaStream_t s);
 cudaError_t launch_ver(const vamrt_projector *p, const void *dose, vamrt_dtype dt, const float *target,
                        long long *out3, cudaStream_t s);
 
@@ -225,10 +237,10 @@ cudaError_t nn_absmax(const float *x, int64_t n, float *out, cudaStream_t s);
 cudaError_t launch_export_u8(const vamrt_projector *p, const void *proj, vamrt_dtype dt, unsigned char *codes,
                              float *dequant, double *clip, cudaStream_t s);
 
-// osmo.cu
+// osmo.cu; ver3 (NULL: not wanted): the voxel error rate of the dose written, as launch_ver's out3
 cudaError_t launch_sum(const vamrt_projector *p, const float *x, double *out, cudaStream_t s);
 cudaError_t launch_osmo_step(const vamrt_projector *p, const float *target, float *model, void *dose,
                              vamrt_dtype dose_dt, const double *fsum, double *err_out, int residual, float alpha,
-                             float mu, float *prev, cudaStream_t s);
+                             float mu, float *prev, long long *ver3, cudaStream_t s);
 
 }  // namespace vamrt

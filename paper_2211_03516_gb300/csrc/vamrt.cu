@@ -156,7 +156,8 @@ void release(vamrt_projector *p)
     cudaFree(p->pad_bricks);
     cudaFree(p->red);
     cudaFree(p->hist);
-    cudaFree(p->dmax);
+    cudaFree(p->ver);
+    cudaFree(p->spans);
     cudaFree(p->ring_vols);
     cudaFree(p->ring_bricks);
     cudaFree(p->ring_cs);
@@ -358,7 +359,9 @@ vamrt_status vamrt_make_projector(const vamrt_geometry *geom, void *stream, vamr
     CK(cudaMalloc(&p->pad_bricks, (size_t)bricks), "cudaMalloc(bricks)");
     CK(cudaMalloc(&p->red, sizeof(double) * (vamrt::kRedBlocks + 8)), "cudaMalloc(reduction)");
     CK(cudaMalloc(&p->hist, sizeof(double) * vamrt::kMaxHistory), "cudaMalloc(history)");
-    CK(cudaMalloc(&p->dmax, sizeof(float) * 4), "cudaMalloc(dmax)");
+    CK(cudaMalloc(&p->ver, sizeof(vamrt::VerState)), "cudaMalloc(error rate)");
+    CK(cudaMalloc(&p->spans, sizeof(int2) * g.ny), "cudaMalloc(resin rows)");
+    CK(vamrt::launch_resin_spans(p, s), "resin rows");
     CK(cudaMallocHost(&p->host_err, 4 * sizeof(double)), "cudaMallocHost");   // E and the 3 VER counts
     p->device_bytes = (sizeof(double4_32a) * 2 + sizeof(int2)) * (uint64_t)p->n_rays + sizeof(double2) * g.n_angles +
                       sizeof(float) * (uint64_t)p->pad_elems;
@@ -696,9 +699,11 @@ vamrt_status vamrt_optimize(vamrt_projector *p, const float *target, float *mode
         // d = A g (left in the scratch volume), then normalise, update, error
         CK(dose_in_scratch(p, proj, params->proj_dtype, s), "forward kernels");
         if (params->timing) CK(cudaEventRecord(ev[2], s), "cudaEventRecord");
+        // a checked iteration's voxel error rate comes from the same pass over the dose
+        const bool check = (it + 1) % params->check_every == 0 || it + 1 == params->max_iter;
         CK(vamrt::launch_osmo_step(p, target, model, dose, params->dose_dtype, fsum, p->hist + it, proj_space ? 1 : 0,
                                    (float)step, (float)params->momentum,
-                                   params->momentum != 0.0 ? params->prev_model : nullptr, s),
+                                   params->momentum != 0.0 ? params->prev_model : nullptr, check ? ver3 : nullptr, s),
            "osmo step");
         if (proj_space) {
             // g <- max(0, g + A^T (f - dn)); the residual is in the model buffer
@@ -715,9 +720,8 @@ vamrt_status vamrt_optimize(vamrt_projector *p, const float *target, float *mode
             t_upd += ms[2];
         }
         ++it;
-        if (it % params->check_every == 0 || it == params->max_iter) {
-            // the voxel error rate of this iteration's normalised dose, then E and V together
-            CK(vamrt::launch_ver(p, dose, params->dose_dtype, target, ver3, s), "voxel error rate kernels");
+        if (check) {
+            // E and the voxel error rate of this iteration's normalised dose together
             CK(cudaMemcpyAsync(&host_chk->err, p->hist + it - 1, sizeof(double), cudaMemcpyDeviceToHost, s), "copy");
             CK(cudaMemcpyAsync(host_chk->ver3, ver3, 3 * sizeof(long long), cudaMemcpyDeviceToHost, s), "copy");
             CK(cudaStreamSynchronize(s), "sync");
