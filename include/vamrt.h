@@ -397,6 +397,13 @@ vamrt_status vamrt_conv3d_tiling(int32_t d, int32_t h, int32_t wd, int32_t cin, 
  *   per X box), nstage, cwA, cwB (channels per column block of X and dy), slots,
  *   slot_bytes, per_sm (blocks per SM), ncols (TMEM), ngroups, nsplit, spb (stages per
  *   block)}.
+ * vamrt_conv3d_wgrad_halo_plan: out[20] = {planned (0: the kernel of the plan above takes the
+ *   shape), TZ, TY, XB (planes, rows, columns per tile), cg (16-channel chunks of x per
+ *   block), ngroups (of chunks), Ct (output channels per block), nslices (of them), nt (M
+ *   tiles), kp (accumulators per M tile), slots, slot_bytes, x_bytes (a slot's part of x),
+ *   ncols (TMEM), nsplit (blocks along the tiles), nx, ny (tiles along x and y), ntiles, seg
+ *   (tiles between two additions into dw), run (positions per block, one after another; 0:
+ *   every nsplit-th tile)}.
  * Errors: EINVAL (NULL out, sms < 1, empty volume); an unsupported shape returns VAMRT_OK
  * with out[0] = 0.
  */
@@ -404,6 +411,8 @@ vamrt_status vamrt_conv3d_halo_plan(int32_t d, int32_t h, int32_t wd, int32_t ci
                                     int32_t sms, int32_t *out);
 vamrt_status vamrt_conv3d_wgrad_plan(int32_t d, int32_t h, int32_t wd, int32_t cin, int32_t cout, int32_t taps,
                                      int32_t sms, int32_t *out);
+vamrt_status vamrt_conv3d_wgrad_halo_plan(int32_t d, int32_t h, int32_t wd, int32_t cin, int32_t cout, int32_t taps,
+                                          int32_t sms, int32_t *out);
 
 
 /*
@@ -413,7 +422,7 @@ vamrt_status vamrt_conv3d_wgrad_plan(int32_t d, int32_t h, int32_t wd, int32_t c
  *
  * vamrt_conv3d_wgrad_bf16: dw[co][t][ci] += sum_p dy[p][co] x[p + off(t)][ci] for the
  *   convolution of vamrt_conv3d_bf16 (same x layout; dy [d][h][wd][cout]); tensor cores
- *   (rows t cin + ci in M, cout in N, positions in K; operands loaded by TMA), split over
+ *   (taps and cin in M, cout in N, positions in K; operands loaded by TMA), split over
  *   positions with FP32 atomics (caller zeroes dw).  wd a multiple of 16, d h wd < 2^31,
  *   cin 16..1024, cout 16..256; x and dy 16-byte aligned.
  * vamrt_nn_resample: op 0 = 2x2x2 average pool (fine -> coarse), 1 = its backward (coarse

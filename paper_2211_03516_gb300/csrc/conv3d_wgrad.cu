@@ -8,7 +8,8 @@
 // a range of positions walked in stages of KS; at the end it adds its partial sums into
 // dW with FP32 atomics (consecutive lanes = consecutive rows t Cin + ci: coalesced).
 // Every wait is bounded (2 s): on timeout the block sets the error flag, waits (bounded)
-// for its own MMAs, frees its TMEM and returns.
+// for its own MMAs, frees its TMEM and returns.  Narrow 3x3x3 layers take the kernel of
+// conv3d_wgrad_halo.cu, whose plan says which.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <cuda_bf16.h>
@@ -358,7 +359,12 @@ PFN_cuTensorMapEncodeTiled_v12000 tma_encoder()
 cudaError_t launch_conv3d_wgrad_tc(const void *X, const void *dY, float *dW, int D, int H, int W, int Cin, int Cout,
                                    int taps, int *err, cudaStream_t s)
 {
-    const cudaError_t e = launch_wgrad_tma(X, dY, dW, D, H, W, Cin, Cout, taps, err, s);
+    WgradHaloPlan pl;
+    cudaError_t e = cudaErrorNotSupported;
+    if (!(((uintptr_t)X | (uintptr_t)dY) & 15) && plan_wgrad_halo(D, H, W, Cin, Cout, taps, sm_count_wgrad(), &pl))
+        e = launch_wgrad_halo(X, dY, dW, D, H, W, Cin, Cout, pl, err, s);
+    else
+        e = launch_wgrad_tma(X, dY, dW, D, H, W, Cin, Cout, taps, err, s);
     if (e == cudaSuccess) count_launches(1);
     return e;
 }

@@ -200,6 +200,16 @@ struct WgradPlan {
 };
 bool plan_wgrad_tma(int D, int H, int W, int Cin, int Cout, int taps, int sms, WgradPlan *pl);
 
+// conv3d_wgrad_halo.cu: plan and launch of the weight gradient that stages each tile of X once
+// for all 27 taps (host only; false for shapes it cannot take)
+struct WgradHaloPlan {
+    int TZ, TY, XB, cg, ngroups, Ct, nslices, nt, kp, slots, slot_bytes, x_bytes, ncols, nsplit, nx, ny, ntiles, seg, run,
+        npos;
+};
+bool plan_wgrad_halo(int D, int H, int W, int Cin, int Cout, int taps, int sms, WgradHaloPlan *pl);
+cudaError_t launch_wgrad_halo(const void *X, const void *dY, float *dW, int D, int H, int W, int Cin, int Cout,
+                              const WgradHaloPlan &pl, int *err, cudaStream_t s);
+
 // conv3d_wgrad.cu: the driver's tensor-map encoder (cuTensorMapEncodeTiled, through the
 // runtime's driver entry point); NULL when the driver does not provide it
 PFN_cuTensorMapEncodeTiled_v12000 tma_encoder();

@@ -62,6 +62,19 @@ vamrt_status vamrt_conv3d_wgrad_plan(int32_t d, int32_t h, int32_t wd, int32_t c
     return VAMRT_OK;
 }
 
+vamrt_status vamrt_conv3d_wgrad_halo_plan(int32_t d, int32_t h, int32_t wd, int32_t cin, int32_t cout, int32_t taps,
+                                          int32_t sms, int32_t *out)
+{
+    if (!out || sms < 1 || d < 1 || h < 1 || wd < 1) return einval("NULL out, sms < 1 or empty volume");
+    vamrt::WgradHaloPlan pl;
+    for (int i = 0; i < 20; ++i) out[i] = 0;
+    if (!vamrt::plan_wgrad_halo(d, h, wd, cin, cout, taps, sms, &pl)) return VAMRT_OK;
+    const int32_t v[20] = {1, pl.TZ, pl.TY, pl.XB, pl.cg, pl.ngroups, pl.Ct, pl.nslices, pl.nt, pl.kp, pl.slots,
+                           pl.slot_bytes, pl.x_bytes, pl.ncols, pl.nsplit, pl.nx, pl.ny, pl.ntiles, pl.seg, pl.run};
+    for (int i = 0; i < 20; ++i) out[i] = v[i];
+    return VAMRT_OK;
+}
+
 vamrt_status vamrt_nn_resample(int32_t op, const void *in, void *out, int32_t d, int32_t h, int32_t w, int32_t c,
                                void *stream)
 {

@@ -81,6 +81,20 @@ static __device__ __forceinline__ uint32_t instr_desc(int m, int n)
     return d;
 }
 
+// true in one lane of a converged warp (the same lane every time)
+static __device__ __forceinline__ bool elect_one()
+{
+    uint32_t r;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "elect.sync _|p, 0xffffffff;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(r)
+        :
+        : "memory");
+    return r != 0;
+}
+
 static __device__ __forceinline__ void mma_bf16(uint32_t tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc)
 {
     asm volatile(
