@@ -374,10 +374,11 @@ vamrt_status vamrt_ramlak_filter(const float *proj, float *out, int64_t rows, in
                                  uint32_t flags, void *stream);
 
 /*
- * vamrt_conv3d_tiling: which kernel vamrt_conv3d_bf16 runs for this shape on the current
- * device, written to out[4] (host array): out[0] = 1 for the halo-tile kernel (W % 8 == 0
- * and W <= 240, x 16-byte aligned at run time; regions of out[1] planes x out[2] rows,
- * out[3] output channels per work item), 0 for the
+ * vamrt_conv3d_tiling: which kernels vamrt_conv3d_bf16 has for this shape on the current
+ * device, written to out[4] (host array): out[0] = 1 for those that stage input tiles by TMA (W %
+ * 8 == 0 and W <= 240, x 16-byte aligned at run time; the halo-tile kernel's regions of out[1]
+ * planes x out[2] rows, out[3] output channels per work item, which the kernel of
+ * vamrt_conv3d_march_plan replaces for the shapes that it takes), 0 for the
  * gather kernel (out[1..3] = 0).  Host-only query, launches nothing.  Errors: EINVAL (NULL or
  * sizes vamrt_conv3d_bf16 rejects), ECUDA (no device).
  */
@@ -392,6 +393,10 @@ vamrt_status vamrt_conv3d_tiling(int32_t d, int32_t h, int32_t wd, int32_t cin, 
  *   row), PT (slots per staged plane), NX (dx taps stacked in N), rowtile, mg (margin
  *   rows), adv (slots between tiles), a_bytes (staged input tile with slack), box_bytes
  *   (its TMA box), stage_bytes, ncols (TMEM), ry (regions along y), nslice, nitems}.
+ * vamrt_conv3d_march_plan: out[12] = {planned (0: the kernel of the plan above takes the
+ *   shape), T (tiles of 128 slots per block), TY (rows of them), mg (margin slots), adv (slots
+ *   between tiles), ncols (TMEM), box_bytes (a 16-channel chunk of a plane of x), stage_bytes,
+ *   ns (stages), nslice (of 16 output channels), ry (columns of rows), nblk (blocks per slice)}.
  * vamrt_conv3d_wgrad_plan: out[17] = {planned, Mtot (taps x cin), nmt (M tiles), tpg
  *   (tiles per group), kp (accumulators per tile), KS (positions per stage), BX (positions
  *   per X box), nstage, cwA, cwB (channels per column block of X and dy), slots,
@@ -409,6 +414,8 @@ vamrt_status vamrt_conv3d_tiling(int32_t d, int32_t h, int32_t wd, int32_t cin, 
  */
 vamrt_status vamrt_conv3d_halo_plan(int32_t d, int32_t h, int32_t wd, int32_t cin, int32_t cout, int32_t taps,
                                     int32_t sms, int32_t *out);
+vamrt_status vamrt_conv3d_march_plan(int32_t d, int32_t h, int32_t wd, int32_t cin, int32_t cout, int32_t taps,
+                                     int32_t sms, int32_t *out);
 vamrt_status vamrt_conv3d_wgrad_plan(int32_t d, int32_t h, int32_t wd, int32_t cin, int32_t cout, int32_t taps,
                                      int32_t sms, int32_t *out);
 vamrt_status vamrt_conv3d_wgrad_halo_plan(int32_t d, int32_t h, int32_t wd, int32_t cin, int32_t cout, int32_t taps,

@@ -44,6 +44,7 @@
 #include <cuda_bf16.h>
 #include <stdint.h>
 
+#include "conv_epilogue.cuh"
 #include "internal.cuh"
 #include "tcgen05.cuh"
 
@@ -84,15 +85,6 @@ __device__ void halo_fail(volatile int *abort_flag, int *err)
 __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes)
 {
     asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap *map, int c0, int c1, int c2, int c3,
-                                            uint32_t bar)
-{
-    asm volatile(
-        "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, "
-        "%5}], [%6];" ::"r"(dst),
-        "l"((uint64_t)map), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(bar)
-        : "memory");
 }
 
 // warps 4-7: per 16-channel chunk, one TMA box of the input tile (thread 0 adds its byte
@@ -155,7 +147,7 @@ __device__ void role_mma(const HaloArgs &a, int k0, uint32_t sbase, uint32_t tme
     int i = 0, k = 0;
     for (int item = blockIdx.x; item < a.nitems; item += gridDim.x, ++k) {
         const int b = k & 1;
-        if (k >= 2 && !mbar_wait(acce0 + 8 * b, ((k >> 1) - 1) & 1)) {
+        if (k >= 2 && !__all_sync(0xffffffffu, mbar_wait(acce0 + 8 * b, ((k >> 1) - 1) & 1))) {
             halo_fail(abort_flag, a.err);
             return;
         }
@@ -163,7 +155,7 @@ __device__ void role_mma(const HaloArgs &a, int k0, uint32_t sbase, uint32_t tme
         const uint32_t dcol = tmem + (uint32_t)(b * a.T * NN);
         for (int c = 0; c < nc; ++c, ++i) {
             const int s = i & 1;
-            if (!mbar_wait(full0 + 8 * s, (i >> 1) & 1) || *abort_flag) {
+            if (!__all_sync(0xffffffffu, mbar_wait(full0 + 8 * s, (i >> 1) & 1) && !*abort_flag)) {
                 halo_fail(abort_flag, a.err);
                 return;
             }
@@ -178,63 +170,13 @@ __device__ void role_mma(const HaloArgs &a, int k0, uint32_t sbase, uint32_t tme
                 const uint32_t acc = (c | g) ? 1u : 0u;
                 uint32_t d = dcol + (uint32_t)(k0 * NN);
                 for (int j = k0; j < a.T; j += kMmaWarps, d += (uint32_t)(kMmaWarps * NN))
-                    mma_bf16(d, (uint64_t)((int64_t)s_adesc[j] + dt), bdesc, idesc, acc);
+                    if (elect_one()) mma_bf16(d, (uint64_t)((int64_t)s_adesc[j] + dt), bdesc, idesc, acc);
             }
-            mma_commit(empty0 + 8 * s);
+            if (elect_one()) mma_commit(empty0 + 8 * s);
         }
-        mma_commit(accf0 + 8 * b);
+        if (elect_one()) mma_commit(accf0 + 8 * b);
     }
 }
-
-template <typename OT>
-__device__ __forceinline__ void store16(OT *dst, const uint32_t *v, const float *bias, int relu)
-{
-    float r[16];
-#pragma unroll
-    for (int i = 0; i < 16; i += 4) {
-        const float4 b4 = bias ? __ldg((const float4 *)(bias + i)) : make_float4(0.f, 0.f, 0.f, 0.f);
-        r[i] = __uint_as_float(v[i]) + b4.x;
-        r[i + 1] = __uint_as_float(v[i + 1]) + b4.y;
-        r[i + 2] = __uint_as_float(v[i + 2]) + b4.z;
-        r[i + 3] = __uint_as_float(v[i + 3]) + b4.w;
-    }
-    if (relu) {
-#pragma unroll
-        for (int i = 0; i < 16; ++i) r[i] = fmaxf(r[i], 0.f);
-    }
-    if constexpr (sizeof(OT) == 2) {
-        uint32_t p[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const __nv_bfloat162 h = __floats2bfloat162_rn(r[2 * i], r[2 * i + 1]);
-            p[i] = *(const uint32_t *)&h;
-        }
-        uint4 *d = (uint4 *)dst;
-        d[0] = make_uint4(p[0], p[1], p[2], p[3]);
-        d[1] = make_uint4(p[4], p[5], p[6], p[7]);
-    } else {
-        float4 *d = (float4 *)dst;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) d[i] = make_float4(r[4 * i], r[4 * i + 1], r[4 * i + 2], r[4 * i + 3]);
-    }
-}
-
-// the 128 threads of epilogue set `set` (warps 4 set .. 4 set + 3) agree on a flag
-// (named barrier 1 + set)
-__device__ __forceinline__ bool epi_all(bool v, int set)
-{
-    uint32_t r;
-    asm volatile(
-        "{\n\t.reg .pred p, q;\n\t"
-        "setp.ne.b32 p, %1, 0;\n\t"
-        "bar.red.and.pred q, %2, 128, p;\n\t"
-        "selp.u32 %0, 1, 0, q;\n\t}"
-        : "=r"(r)
-        : "r"((uint32_t)v), "r"(1 + set)
-        : "memory");
-    return r != 0;
-}
-__device__ __forceinline__ void epi_sync(int set) { asm volatile("bar.sync %0, 128;" ::"r"(1 + set) : "memory"); }
 
 // warps 0-7: TMEM -> Y, two sets of four warps taking alternate tiles (warp 4 s + w of set
 // s reads TMEM lane quarter w).  Row m of a tile holds, for each dx, the (dz, dy)-summed
@@ -377,8 +319,8 @@ __global__ void __launch_bounds__(kHaloThreads, 1)
         role_epilogue<OT>(a, tmem, s_q, s_oz, s_xch, accf0, acce0, &s_abort);
     else if (warp < kMmaWarp0)
         role_load<TAPS>(&xmap, a, sbase, full0, empty0, &s_abort);
-    else if ((tid & 31) == 0)
-        role_mma<TAPS>(a, warp - kMmaWarp0, sbase, tmem, s_adesc, full0, empty0, accf0, acce0, &s_abort);
+    else
+        role_mma<TAPS>(a, __shfl_sync(0xffffffffu, warp - kMmaWarp0, 0), sbase, tmem, s_adesc, full0, empty0, accf0, acce0, &s_abort);
 
     tc_fence_before();
     __syncthreads();

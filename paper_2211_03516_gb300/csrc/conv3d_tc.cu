@@ -164,13 +164,29 @@ __global__ void __launch_bounds__(kConvThreads)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ncols) : "memory");
 }
 
+int device_sms()
+{
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return 0;
+    return n;
+}
+
 }  // namespace
 
 cudaError_t launch_conv3d_tc(const void *X, const void *Wt, const float *bias, void *Y, int out_f32, int D, int H,
                              int W, int Cin, int Cout, int taps, int relu, int *err, cudaStream_t s)
 {
-    // the halo-tile kernel takes every shape with W % 8 == 0; this gather kernel the rest
-    cudaError_t e = launch_conv3d_halo(X, Wt, bias, Y, out_f32, D, H, W, Cin, Cout, taps, relu, err, s);
+    // 3x3x3 layers walk along z where that kernel's weights fit beside its stages: faster than the
+    // halo-tile kernel on every layer timed (us, halo-tile -> walk: 46 x 32 x 32 32 -> 64 33 -> 20, 192 -> 64
+    // 121 -> 64, 23 x 16 x 16 64 -> 128 29 -> 18, 184 x 128 x 128 48 -> 16 283 -> 160)
+    ConvMarchPlan mp;
+    cudaError_t e = cudaErrorNotSupported;
+    if (plan_conv3d_march(D, H, W, Cin, Cout, taps, device_sms(), &mp))
+        e = launch_conv3d_march(X, Wt, bias, Y, out_f32, D, H, W, Cin, Cout, relu, mp, err, s);
+    if (e != cudaErrorNotSupported) return e;
+    // the halo-tile kernel takes every other shape with W % 8 == 0; this gather kernel the rest
+    e = launch_conv3d_halo(X, Wt, bias, Y, out_f32, D, H, W, Cin, Cout, taps, relu, err, s);
     if (e != cudaErrorNotSupported) return e;
     const int64_t P = (int64_t)D * H * W;
     const unsigned grid = (unsigned)((P + kM - 1) / kM);

@@ -64,10 +64,6 @@ struct Args {
     int Cin;
 };
 
-__device__ __forceinline__ void arrive_expect_tx(uint32_t bar, uint32_t bytes)
-{
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
 // box at channel 0 of slot (x, y) and the outer coordinates u, v
 __device__ __forceinline__ void load_box(uint32_t dst, const CUtensorMap *map, int x, int y, int u, int v, uint32_t bar)
 {
@@ -172,7 +168,7 @@ __global__ void __launch_bounds__(kWgThreads, 1)
                 break;
             }
             const uint32_t sb = base + slot * p.slot_bytes, bar = full0 + 8 * slot;
-            if (lane == 0) arrive_expect_tx(bar, (uint32_t)(p.x_bytes + 3 * nb * ybytes));
+            if (lane == 0) mbar_arrive_expect_tx(bar, (uint32_t)(p.x_bytes + 3 * nb * ybytes));
             __syncwarp();
             const int tx = tile % p.nx, r = tile / p.nx, ty = r % p.ny, tz = r / p.ny;
             if (lane == 0)

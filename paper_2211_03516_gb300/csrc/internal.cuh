@@ -214,6 +214,14 @@ cudaError_t launch_wgrad_halo(const void *X, const void *dY, float *dW, int D, i
 // runtime's driver entry point); NULL when the driver does not provide it
 PFN_cuTensorMapEncodeTiled_v12000 tma_encoder();
 
+// conv3d_march.cu (blocks walk along z; 3x3x3): plan (false for shapes it does not take), launch
+struct ConvMarchPlan {
+    int T, TY, mg, adv, ncols, box_bytes, stage_bytes, ns, nslice, ry, nblk;
+};
+bool plan_conv3d_march(int D, int H, int W, int Cin, int Cout, int taps, int sms, ConvMarchPlan *pl);
+cudaError_t launch_conv3d_march(const void *X, const void *Wt, const float *bias, void *Y, int out_f32, int D, int H,
+                                int W, int Cin, int Cout, int relu, const ConvMarchPlan &pl, int *err, cudaStream_t s);
+
 // conv3d_halo.cu (persistent halo-tile variant; W % 8 == 0).  launch returns
 // cudaErrorNotSupported for shapes it does not take.
 struct ConvHaloPlan {

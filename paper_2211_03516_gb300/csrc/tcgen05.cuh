@@ -2,6 +2,7 @@
 // waits, shared-memory matrix descriptors, tcgen05 MMA / commit / TMEM loads, cp.async
 // copies.  sm_100-family only.
 #pragma once
+#include <cuda.h>
 #include <stdint.h>
 
 namespace vamrt {
@@ -54,6 +55,21 @@ static __device__ __noinline__ bool mbar_wait(uint32_t bar, uint32_t parity)
 static __device__ __forceinline__ void mbar_arrive(uint32_t bar)
 {
     asm volatile("mbarrier.arrive.release.cta.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+
+// arrive and raise the phase's expected transaction bytes
+static __device__ __forceinline__ void mbar_arrive_expect_tx(uint32_t bar, uint32_t bytes)
+{
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
+static __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap *map, int c0, int c1, int c2, int c3,
+                                                   uint32_t bar)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, "
+        "%5}], [%6];" ::"r"(dst),
+        "l"((uint64_t)map), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(bar)
+        : "memory");
 }
 
 // Shared-memory matrix descriptor, no swizzle, K-major: lbo = byte distance between the
