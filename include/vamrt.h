@@ -393,10 +393,10 @@ vamrt_status vamrt_conv3d_tiling(int32_t d, int32_t h, int32_t wd, int32_t cin, 
  *   row), PT (slots per staged plane), NX (dx taps stacked in N), rowtile, mg (margin
  *   rows), adv (slots between tiles), a_bytes (staged input tile with slack), box_bytes
  *   (its TMA box), stage_bytes, ncols (TMEM), ry (regions along y), nslice, nitems}.
- * vamrt_conv3d_march_plan: out[12] = {planned (0: the kernel of the plan above takes the
+ * vamrt_conv3d_march_plan: out[13] = {planned (0: the kernel of the plan above takes the
  *   shape), T (tiles of 128 slots per block), TY (rows of them), mg (margin slots), adv (slots
- *   between tiles), ncols (TMEM), box_bytes (a 16-channel chunk of a plane of x), stage_bytes,
- *   ns (stages), nslice (of 16 output channels), ry (columns of rows), nblk (blocks per slice)}.
+ *   between tiles), ncols (TMEM), cps (16-channel chunks per stage), box_bytes (those chunks of
+ *   a plane of x), stage_bytes, ns (stages), nslice (of 16 output channels), ry (columns of rows), nblk (blocks per slice)}.
  * vamrt_conv3d_wgrad_plan: out[17] = {planned, Mtot (taps x cin), nmt (M tiles), tpg
  *   (tiles per group), kp (accumulators per tile), KS (positions per stage), BX (positions
  *   per X box), nstage, cwA, cwB (channels per column block of X and dy), slots,

@@ -8,10 +8,10 @@
 // (32 cycles at 128 bytes a cycle) for N = 48 columns (24 cycles of tensor work).
 //
 // A block takes TY rows x all W columns (T <= 2 tiles of 128 slots) of one 16-channel slice of Y,
-// keeps that slice's weights in shared memory, and walks z.  A stage is one 16-channel chunk of
-// one plane of X with one halo row on either side: (TY + 2) x W slots of 32 bytes in the 32-byte
-// swizzled K-major layout, one TMA box, zero fill outside the volume.  The chunk's A operand for
-// dy is the slot run shifted by whole rows.  N stacks (output plane, dx, co): the plane z' adds to
+// keeps that slice's weights in shared memory, and walks z.  A stage is cps (1, 2 or 4) 16-channel
+// chunks of one plane of X with one halo row on either side: (TY + 2) x W slots of 32, 64 or 128
+// bytes in the swizzled K-major layout of that width, one TMA box, zero fill outside the volume
+// and past the last channel.  A chunk's A operand for dy is the slot run shifted by whole rows.  N stacks (output plane, dx, co): the plane z' adds to
 // the outputs z' - 1, z' and z' + 1, whose accumulators (48 columns each: three dx x 16) stand
 // side by side in a ring of kRing planes per tile, so one MMA has N = 144 (two where the ring
 // wraps; the first MMA into a new plane overwrites and goes apart).  The epilogue adds the dx
@@ -19,9 +19,12 @@
 // a row's ends left out.  Where W does not divide 128, tiles run through the rows 120 slots
 // apart with a margin slot at either end, starting 8 slots ahead of the first row.
 //
-// Measured (GB300, us, conv3d_halo.cu -> this kernel): 48 -> 16 channels on 184 x 128 x 128 283 -> 160
-// (780 TFLOP/s), 16 -> 48 there 342 -> 244, 16 -> 16 123 -> 91, 96 -> 32 on 92 x 64 x 64 199 -> 81, 192 ->
-// 64 on 46 x 32 x 32 121 -> 64.
+// Measured (GB300, us, conv3d_halo.cu -> this kernel with 32-byte slots -> with the widest slots): 48 ->
+// 16 channels on 184 x 128 x 128 283 -> 160 -> 140 (893 TFLOP/s), 16 -> 48 there 342 -> 244 -> 240, 16 ->
+// 16 123 -> 91 -> 89, 96 -> 32 on 92 x 64 x 64 199 -> 81 -> 69, 192 -> 64 on 46 x 32 x 32 121 -> 64 -> 56, 64 ->
+// 64 there 50 -> 27 -> 22.  Wide operand rows are read faster and take fewer stages.  What bounds it
+// now (48 -> 16): the MMAs (145 us without the epilogue's arithmetic and 160 with it, at 32-byte
+// slots); TMA and the stores do not show.
 //
 // Roles: kMarchSets sets of 4 epilogue warps take (plane, tile) units in turn, one warp issues the
 // TMA boxes, and one warp per tile issues its MMAs (one elected lane; the order of the MMAs into
@@ -44,9 +47,8 @@ constexpr int kMarchSets = 4, kMarchLoad = 4 * kMarchSets, kMarchMma = kMarchLoa
 constexpr int kMarchThreads = 32 * (kMarchMma + kMaxT);
 constexpr int kRing = 5;                    // output planes per tile in TMEM
 constexpr int kMaxStages = 8;
-constexpr int kSlot = 32;                   // bytes of a slot: 16 BF16 channels of one voxel
-constexpr int kLead = 256;                  // bytes ahead of a stage's box (8 slots)
-constexpr int kWBytes = 27 * 16 * kSlot;    // weights of one chunk: [dy][144 rows][16]
+constexpr int kLead = 8;                    // slots ahead of a stage's box
+constexpr int kWBytes = 27 * 16 * 32;       // weights of one chunk: [dy][144 rows][16]
 constexpr int kMarchSmem = 220 * 1024;
 
 struct MarchArgs {
@@ -143,7 +145,7 @@ __device__ void march_epilogue(const MarchArgs &a, uint32_t tmem, int l0, int l1
     }
 }
 
-template <typename OT>
+template <typename OT, int CPS>
 __global__ void __launch_bounds__(kMarchThreads, 1)
     conv3d_march_kernel(const __grid_constant__ CUtensorMap xmap, const MarchArgs a)
 {
@@ -157,6 +159,7 @@ __global__ void __launch_bounds__(kMarchThreads, 1)
     const ConvMarchPlan &p = a.p;
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int slice = blockIdx.x % p.nslice, co0 = 16 * slice, nc = a.Cin >> 4;
+    constexpr int sb = 32 * CPS;           // bytes of a slot
     const int64_t tot = (int64_t)p.ry * a.D, blk = blockIdx.x / p.nslice;
     const int l0 = (int)(blk * tot / p.nblk), l1 = (int)((blk + 1) * tot / p.nblk);
     const uint32_t sbase = smem_u32(smem), wbase = sbase, xbase = sbase + nc * kWBytes;
@@ -181,7 +184,7 @@ __global__ void __launch_bounds__(kMarchThreads, 1)
         const int h = i & 1, n = (i >> 1) % 144, cd = (i >> 1) / 144, dy = cd % 3, c = cd / 3;
         const int b = n / 48, dx = n / 16 % 3, co = n & 15, tap = (2 - b) * 9 + dy * 3 + dx;
         const uint4 w = *(const uint4 *)(a.Wt + ((int64_t)(co0 + co) * 27 + tap) * a.Cin + c * 16 + h * 8);
-        *(uint4 *)(smem + c * kWBytes + dy * 144 * kSlot + (n >> 3) * 256 + h * 128 + (n & 7) * 16) = w;
+        *(uint4 *)(smem + c * kWBytes + dy * 144 * 32 + (n >> 3) * 256 + h * 128 + (n & 7) * 16) = w;
     }
     fence_proxy_async();
     tc_fence_before();
@@ -197,13 +200,13 @@ __global__ void __launch_bounds__(kMarchThreads, 1)
         for (int l = l0; l < l1 && ok;) {
             const Piece pc = piece_at(a, l, l1);
             for (int z = pc.z0 - 1; z <= pc.z1 && ok; ++z)
-                for (int c = 0; c < nc; ++c, ++i) {
+                for (int c = 0; c < nc; c += CPS, ++i) {
                     if (i >= p.ns) ok = mbar_wait(empty + 8 * s, phase);
                     ok = __all_sync(0xffffffffu, ok && !s_abort);
                     if (!ok) break;
                     if (lane == 0) {
                         mbar_arrive_expect_tx(full + 8 * s, (uint32_t)p.box_bytes);
-                        tma_load_4d(xbase + s * p.stage_bytes + kLead, &xmap, c * 16, 0, pc.y0 - 1, z, full + 8 * s);
+                        tma_load_4d(xbase + s * p.stage_bytes + kLead * sb, &xmap, c * 16, 0, pc.y0 - 1, z, full + 8 * s);
                     }
                     __syncwarp();
                     if (++s == p.ns) {
@@ -217,7 +220,8 @@ __global__ void __launch_bounds__(kMarchThreads, 1)
     } else if (warp - kMarchMma < p.T) {
         const int t = warp - kMarchMma;
         const uint32_t dcol = tmem + (uint32_t)(t * kRing * 48);
-        const uint64_t sw = (uint64_t)6 << 61;
+        const uint64_t sw = (uint64_t)(CPS == 4 ? 2 : CPS == 2 ? 4 : 6) << 61;
+        const int row16 = a.W * sb / 16;          // a row, in descriptor units of 16 bytes
         int s = 0, phase = 0, g = 0;
         bool ok = true;
         for (int l = l0; l < l1 && ok;) {
@@ -228,31 +232,41 @@ __global__ void __launch_bounds__(kMarchThreads, 1)
                 const int lo = max(z - 1, pc.z0), hi = min(z + 1, pc.z1 - 1), n = hi - lo + 1, b0 = lo - (z - 1);
                 const bool fresh = z + 1 < pc.z1;
                 const int s0 = (g + lo - pc.z0) % kRing, n1 = min(n, kRing - s0);
+                const bool wrap = n > n1;
+                const uint32_t id1 = instr_desc(128, 48 * n1), id2 = instr_desc(128, 48 * (n - n1)), d1 = dcol + s0 * 48;
                 if (fresh) {
                     const int u = g + z + 1 - pc.z0;
                     if (u >= kRing) ok = mbar_wait(acce + 8 * (u % kRing), (u / kRing - 1) & 1);
                 }
-                for (int c = 0; c < nc; ++c) {
+                for (int c = 0; c < nc; c += CPS) {
                     ok = ok && mbar_wait(full + 8 * s, phase);
                     ok = __all_sync(0xffffffffu, ok && !s_abort);
                     if (!ok) break;
                     tc_fence_after();
                     if (elect_one()) {
-                        const uint64_t A = smem_desc(xbase + s * p.stage_bytes + kLead +
-                                                         (p.adv * t - 8 * p.mg) * kSlot, 16, 256) | sw;
-                        const uint64_t B = smem_desc(wbase + c * kWBytes, 128, 256);
+                        const uint64_t A0 = smem_desc(xbase + s * p.stage_bytes +
+                                                          (kLead + p.adv * t - 8 * p.mg) * sb, 16, 8 * sb) | sw;
+                        const uint64_t B0 = smem_desc(wbase + c * kWBytes, 128, 256) + (uint64_t)(b0 * 96);
 #pragma unroll
-                        for (int dy = 0; dy < 3; ++dy) {
-                            const uint64_t Ad = A + (uint64_t)(dy * a.W * (kSlot / 16));
-                            const uint64_t Bd = B + (uint64_t)(dy * 144 * (kSlot / 16) + b0 * 96);
-                            // first MMA of a fresh plane overwrites: it goes apart from the others
-                            const bool apart = fresh && c == 0 && dy == 0;
-                            const int na = apart ? n - 1 : n, n1a = min(n1, na);
-                            if (n1a > 0) mma_bf16(dcol + s0 * 48, Ad, Bd, instr_desc(128, 48 * n1a), 1u);
-                            if (na > n1a) mma_bf16(dcol, Ad, Bd + (uint64_t)(n1a * 96), instr_desc(128, 48 * (na - n1a)), 1u);
-                            if (apart)
-                                mma_bf16(dcol + (s0 + n - 1) % kRing * 48, Ad, Bd + (uint64_t)((n - 1) * 96),
-                                         instr_desc(128, 48), 0u);
+                        for (int k = 0; k < CPS; ++k) {
+                            if (k && c + k >= nc) break;
+                            const uint64_t A = A0 + (uint64_t)(2 * k), B = B0 + (uint64_t)(k * (kWBytes / 16));
+#pragma unroll
+                            for (int dy = 0; dy < 3; ++dy) {
+                                const uint64_t Ad = A + (uint64_t)(dy * row16), Bd = B + (uint64_t)(dy * 144 * 2);
+                                if (k == 0 && dy == 0 && fresh && c == 0) {
+                                    // first MMA of a fresh plane overwrites: it goes apart from the others
+                                    const int na = n - 1, n1a = min(n1, na);
+                                    if (n1a > 0) mma_bf16(d1, Ad, Bd, instr_desc(128, 48 * n1a), 1u);
+                                    if (na > n1a)
+                                        mma_bf16(dcol, Ad, Bd + (uint64_t)(n1a * 96), instr_desc(128, 48 * (na - n1a)), 1u);
+                                    mma_bf16(dcol + (s0 + na) % kRing * 48, Ad, Bd + (uint64_t)(na * 96),
+                                             instr_desc(128, 48), 0u);
+                                } else {
+                                    mma_bf16(d1, Ad, Bd, id1, 1u);
+                                    if (wrap) mma_bf16(dcol, Ad, Bd + (uint64_t)(n1 * 96), id2, 1u);
+                                }
+                            }
                         }
                         mma_commit(empty + 8 * s);
                     }
@@ -302,14 +316,20 @@ bool plan_conv3d_march(int D, int H, int W, int Cin, int Cout, int taps, int sms
     p.TY = std::min(two / W, H);
     if (p.TY < 1) return false;
     p.ncols = p.T * kRing * 48 <= 256 ? 256 : 512;
-    p.box_bytes = (p.TY + 2) * W * kSlot;
-    // slots read: two rows below the first tile's start to the end of the last tile
-    const int reach = kLead + (2 * W + p.adv * (p.T - 1) - 8 * p.mg + 128) * kSlot;
-    p.stage_bytes = (std::max(kLead + p.box_bytes, reach) + 1023) / 1024 * 1024;
-    p.ns = std::min(kMaxStages, (kMarchSmem - Cin / 16 * kWBytes) / p.stage_bytes);
+    // the widest slots that leave two stages of several chunks, or three of one
+    for (p.cps = Cin > 32 ? 4 : Cin / 16; p.cps >= 1; p.cps /= 2) {
+        const int sb = 32 * p.cps;
+        p.box_bytes = (p.TY + 2) * W * sb;
+        // slots read: two rows below the first tile's start to the end of the last tile
+        const int reach = kLead + 2 * W + p.adv * (p.T - 1) - 8 * p.mg + 128;
+        p.stage_bytes = (std::max(kLead * sb + p.box_bytes, reach * sb) + 1023) / 1024 * 1024;
+        p.ns = std::min(kMaxStages, (kMarchSmem - Cin / 16 * kWBytes) / p.stage_bytes);
+        if (p.ns >= (p.cps > 1 ? 2 : 3)) break;
+    }
+    if (!p.cps) return false;
     p.nslice = Cout / 16;
     p.ry = (H + p.TY - 1) / p.TY;
-    if (p.ns < 3 || p.nslice > sms || (int64_t)p.ry * D >= (1ll << 31)) return false;
+    if (p.nslice > sms || (int64_t)p.ry * D >= (1ll << 31)) return false;
     p.nblk = (int)std::min<int64_t>(sms / p.nslice, (int64_t)p.ry * D);
     *pl = p;
     return true;
@@ -323,16 +343,24 @@ cudaError_t launch_conv3d_march(const void *X, const void *Wt, const float *bias
     CUtensorMap xmap;
     const cuuint64_t dims[4] = {(cuuint64_t)Cin, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)D};
     const cuuint64_t strides[3] = {(cuuint64_t)Cin * 2, (cuuint64_t)W * Cin * 2, (cuuint64_t)H * W * Cin * 2};
-    const cuuint32_t box[4] = {16, (cuuint32_t)W, (cuuint32_t)(pl.TY + 2), 1};
+    const cuuint32_t box[4] = {(cuuint32_t)(16 * pl.cps), (cuuint32_t)W, (cuuint32_t)(pl.TY + 2), 1};
     const cuuint32_t one[4] = {1, 1, 1, 1};
     if (enc(&xmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void *>(X), dims, strides, box, one,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_32B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+            CU_TENSOR_MAP_INTERLEAVE_NONE,
+            pl.cps == 4 ? CU_TENSOR_MAP_SWIZZLE_128B : pl.cps == 2 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B,
+            CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return cudaErrorNotSupported;
     const MarchArgs a{(const __nv_bfloat16 *)Wt, bias, Y, err, pl, D, H, W, Cin, Cout, relu};
     // at least 116 KB of shared memory keeps one block per SM, so TMEM is never oversubscribed
     const int smem = std::max(Cin / 16 * kWBytes + pl.ns * pl.stage_bytes, 116 * 1024);
-    auto k = out_f32 ? conv3d_march_kernel<float> : conv3d_march_kernel<__nv_bfloat16>;
+    auto k = conv3d_march_kernel<float, 1>;
+    if (out_f32)
+        k = pl.cps == 4 ? conv3d_march_kernel<float, 4> : pl.cps == 2 ? conv3d_march_kernel<float, 2> : k;
+    else
+        k = pl.cps == 4   ? conv3d_march_kernel<__nv_bfloat16, 4>
+            : pl.cps == 2 ? conv3d_march_kernel<__nv_bfloat16, 2>
+                          : conv3d_march_kernel<__nv_bfloat16, 1>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     k<<<(unsigned)(pl.nslice * pl.nblk), kMarchThreads, smem, s>>>(xmap, a);

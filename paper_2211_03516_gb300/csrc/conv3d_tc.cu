@@ -178,8 +178,8 @@ cudaError_t launch_conv3d_tc(const void *X, const void *Wt, const float *bias, v
                              int W, int Cin, int Cout, int taps, int relu, int *err, cudaStream_t s)
 {
     // 3x3x3 layers walk along z where that kernel's weights fit beside its stages: faster than the
-    // halo-tile kernel on every layer timed (us, halo-tile -> walk: 46 x 32 x 32 32 -> 64 33 -> 20, 192 -> 64
-    // 121 -> 64, 23 x 16 x 16 64 -> 128 29 -> 18, 184 x 128 x 128 48 -> 16 283 -> 160)
+    // halo-tile kernel on every layer timed (us, halo-tile -> walk: 46 x 32 x 32 32 -> 64 33 -> 18, 192 -> 64
+    // 121 -> 56, 23 x 16 x 16 64 -> 128 29 -> 16, 184 x 128 x 128 48 -> 16 283 -> 140)
     ConvMarchPlan mp;
     cudaError_t e = cudaErrorNotSupported;
     if (plan_conv3d_march(D, H, W, Cin, Cout, taps, device_sms(), &mp))

@@ -216,7 +216,7 @@ PFN_cuTensorMapEncodeTiled_v12000 tma_encoder();
 
 // conv3d_march.cu (blocks walk along z; 3x3x3): plan (false for shapes it does not take), launch
 struct ConvMarchPlan {
-    int T, TY, mg, adv, ncols, box_bytes, stage_bytes, ns, nslice, ry, nblk;
+    int T, TY, mg, adv, ncols, cps, box_bytes, stage_bytes, ns, nslice, ry, nblk;
 };
 bool plan_conv3d_march(int D, int H, int W, int Cin, int Cout, int taps, int sms, ConvMarchPlan *pl);
 cudaError_t launch_conv3d_march(const void *X, const void *Wt, const float *bias, void *Y, int out_f32, int D, int H,

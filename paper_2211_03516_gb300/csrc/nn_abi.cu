@@ -54,11 +54,11 @@ vamrt_status vamrt_conv3d_march_plan(int32_t d, int32_t h, int32_t wd, int32_t c
 {
     if (!out || sms < 1 || d < 1 || h < 1 || wd < 1) return einval("NULL out, sms < 1 or empty volume");
     vamrt::ConvMarchPlan pl;
-    for (int i = 0; i < 12; ++i) out[i] = 0;
+    for (int i = 0; i < 13; ++i) out[i] = 0;
     if (!vamrt::plan_conv3d_march(d, h, wd, cin, cout, taps, sms, &pl)) return VAMRT_OK;
-    const int32_t v[12] = {1, pl.T, pl.TY, pl.mg, pl.adv, pl.ncols, pl.box_bytes, pl.stage_bytes, pl.ns, pl.nslice,
+    const int32_t v[13] = {1, pl.T, pl.TY, pl.mg, pl.adv, pl.ncols, pl.cps, pl.box_bytes, pl.stage_bytes, pl.ns, pl.nslice,
                            pl.ry, pl.nblk};
-    for (int i = 0; i < 12; ++i) out[i] = v[i];
+    for (int i = 0; i < 13; ++i) out[i] = v[i];
     return VAMRT_OK;
 }
 

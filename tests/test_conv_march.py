@@ -6,8 +6,9 @@ import numpy as np
 import pytest
 
 SHAPES = [((1, 1, 8), 16, 16), ((4, 5, 16), 32, 16), ((9, 3, 128), 16, 32), ((7, 6, 40), 16, 16), ((3, 17, 64), 16, 16),
-          ((5, 4, 112), 32, 16), ((6, 2, 200), 16, 16), ((13, 9, 80), 16, 16), ((2, 9, 232), 16, 16)]
-PLAN = "T TY mg adv ncols box_bytes stage_bytes ns nslice ry nblk".split()
+          ((5, 4, 112), 32, 16), ((6, 2, 200), 16, 16), ((13, 9, 80), 16, 16), ((2, 9, 232), 16, 16),
+          ((3, 5, 64), 48, 16), ((2, 3, 40), 80, 16)]
+PLAN = "T TY mg adv ncols cps box_bytes stage_bytes ns nslice ry nblk".split()
 RING = 5
 
 
@@ -17,7 +18,7 @@ def _plan(shape, cin, cout, sms, taps=27):
     from paper_2211_03516_gb300 import vamrt
     f = vamrt.lib().vamrt_conv3d_march_plan
     f.argtypes = [ctypes.c_int32] * 7 + [ctypes.c_void_p]
-    out = (ctypes.c_int32 * 12)()
+    out = (ctypes.c_int32 * 13)()
     assert f(*shape, cin, cout, taps, sms, ctypes.addressof(out)) == 0
     return dict(zip(PLAN, list(out)[1:])) if out[0] else None
 
@@ -37,8 +38,9 @@ def test_emulated_on_integers(shape, cin, cout, sms):
     (D, H, W), nc = shape, cin // 16
     T, TY, mg, adv = p["T"], p["TY"], p["mg"], p["adv"]
     assert T * RING * 48 <= p["ncols"] <= 512 and p["nslice"] * p["nblk"] <= sms and p["nslice"] * 16 == cout
-    assert 3 <= p["ns"] <= 8 and nc * 27 * 512 + p["ns"] * p["stage_bytes"] <= 220 * 1024 and p["stage_bytes"] % 1024 == 0
-    assert p["box_bytes"] == (TY + 2) * W * 32 and TY + 2 <= 256 and adv % 8 == 0 and W % 8 == 0
+    sb = 32 * p["cps"]          # bytes of a slot: 16 channels of each of cps chunks
+    assert (2 if p["cps"] > 1 else 3) <= p["ns"] <= 8 and nc * 27 * 512 + p["ns"] * p["stage_bytes"] <= 220 * 1024 and p["stage_bytes"] % 1024 == 0
+    assert p["box_bytes"] == (TY + 2) * W * sb and TY + 2 <= 256 and adv % 8 == 0 and W % 8 == 0
     rng = np.random.default_rng(1)
     x, w = rng.integers(-4, 5, shape + (cin,)), rng.integers(-4, 5, (cout, 27, cin))
     y = np.zeros(shape + (cout,), np.int64)
@@ -55,7 +57,7 @@ def test_emulated_on_integers(shape, cin, cout, sms):
                 lo, hi = max(z - 1, z0), min(z + 1, z1 - 1)
                 n, b0, s0, fresh = hi - lo + 1, lo - (z - 1), (g + lo - z0) % RING, z + 1 < z1
                 for c in range(nc):
-                    stage = np.full((p["stage_bytes"] // 32, 16), 777, np.int64)
+                    stage = np.full((p["stage_bytes"] // sb, 16), 777, np.int64)
                     box = np.zeros((TY + 2, W, 16), np.int64)
                     for r in range(TY + 2):
                         if 0 <= z < D and 0 <= y0 - 1 + r < H:
