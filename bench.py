@@ -546,7 +546,9 @@ def run_gpu(args, rank, world):
     # ---- roofline of the dominant kernel (CUDA events around it, inside the library) ----
     # Both operators stage their per-sample data -- 8 trilinear corner words, 32 B -- in
     # shared memory, so the roofline is shared-memory bandwidth, measured here; the HBM
-    # fraction of the compulsory traffic is reported beside it.
+    # fraction of the compulsory traffic is reported beside it.  (Over groups of angles the
+    # projection reads 16 B per corner for four angles and passes over regions that hold
+    # nothing, so its rate by this count exceeds the roofline.)
     smem_bps = vamrt.vamrt_measure_smem_bandwidth()
     l2_read_bps, l2_red_ops = vamrt.vamrt_measure_l2_rates()
     hbm, peak_kind = peaks()
