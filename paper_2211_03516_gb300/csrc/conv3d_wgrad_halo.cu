@@ -33,9 +33,9 @@
 // 33, 48 -> 16 on 100 x 90 x 80 754 -> 57.  What bounds it now: an MMA of 128 x 48 x 16 takes 77
 // cycles, of which its operands' reads are most.
 //
-// A dY row or plane past the volume is zero, as are x < 0 and x >= W of the shifted copies:
-// they meet real X values there, so a voxel of X that is not finite spoils all 27 taps of its
-// channel and not only those whose window reaches it.
+// A dY row or plane past the volume is zero, as are x < 0 and x >= W of the shifted copies: they
+// meet real X values there, so a voxel on a face of X that is not finite spoils all 27 taps of its
+// channel, as one inside does, and not only those that reach it from within the volume.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <cuda_bf16.h>
