@@ -154,8 +154,10 @@ __global__ void __launch_bounds__(kDoseThreads, kDoseBlocks)
             sign |= __any_sync(kFull, gc[c] < 0.f);
             gc[c] *= scale;
         }
+        // a warp without a negative value may hold -0.0 (a dark pixel, or one below zero that vanishes
+        // when it is weighted), as a bit pattern the lowest integer
 #pragma unroll
-        for (int c = 0; c < S; ++c) gc[c] *= sign ? kSignedScale : kNonNegScale;
+        for (int c = 0; c < S; ++c) gc[c] = sign ? gc[c] * kSignedScale : fabsf(gc[c]) * kNonNegScale;
         const int zpitch = sW.EZ, stages = sW.stages, slab = sW.EX * zpitch, y0 = sW.y0, R_ = sW.R, ring_rows = 2 * R_ + 1;
         auto table = [&](int ya, int yb) {      // warp 0, one lane per row
             for (int y = ya + lane; y <= yb; y += 32) {
