@@ -602,8 +602,9 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSm)
             if (cl < cf) cl = cf;
         }
         const float wray = (FWD && active) ? g * R.w : 0.f;
-        // the warp's shares are all non-negative: the subnormal conversion applies
-        const bool nonneg = FWD && __all_sync(kFull, !(wray < 0.f));
+        // the warp's shares are all non-negative: the subnormal conversion applies (not to -0.0, which
+        // a negative pixel becomes where its weight underflows: as a bit pattern the lowest integer)
+        const bool nonneg = FWD && __all_sync(kFull, __float_as_int(wray) >= 0);
         cf = __reduce_min_sync(kFull, cf);
         cl = __reduce_max_sync(kFull, cl);
         // |weights| >= 0 order like their bit patterns

@@ -1,6 +1,6 @@
-"""Projections whose dark pixels hold -0.0: the dose is that of +0.0.  (Non-negative shares become
-fixed point by their bit pattern, in which -0.0 is the lowest integer.)  Tolerance: 1e-5 relative
-L2, as for every FP32 operator."""
+"""Projections whose dark pixels hold -0.0, or negative values that vanish when they are weighted:
+the dose is that of +0.0.  (Non-negative shares become fixed point by their bit pattern, in which
+-0.0 is the lowest integer.)  Tolerance: 1e-5 relative L2, as for every FP32 operator."""
 import numpy as np
 import pytest
 import torch
@@ -24,7 +24,8 @@ def V():
     return vamrt
 
 
-@pytest.mark.parametrize("dtype,dark", [(torch.float32, -0.0), (torch.bfloat16, -0.0), (torch.float16, -0.0)])
+@pytest.mark.parametrize("dtype,dark", [(torch.float32, -0.0), (torch.bfloat16, -0.0), (torch.float16, -0.0),
+                                        (torch.float32, -1.5e-45)])
 @pytest.mark.parametrize("name", list(SCANS))
 def test_dose_of_dark_pixels_below_zero(V, name, dtype, dark):
     w = SCANS[name]
