@@ -14,6 +14,7 @@
 // 38 us for the maximum's 119 MB and 87 us for the histograms' 356 MB (4.1 TB/s; the bins'
 // shared-memory atomics come next), against 1443, 1455 and 50 us of a pass per voxel with an
 // FP64 test and 64-bit divisions and a serial scan.
+#include "exact_div.cuh"
 #include "resin.cuh"
 
 namespace vamrt {
@@ -50,22 +51,25 @@ struct Group<1, T> {
     __device__ __forceinline__ float operator[](int) const { return ldd(&v); }
 };
 
+// The groups of V voxels of a volume, and the exact divisions that take a group's index to its row and
+// plane (padded voxels, and so the indices, are below 2^31)
+struct Groups {
+    unsigned per, ny, all;       // groups per row, rows per plane, groups
+    ExactDiv by_per, by_ny;
+    Groups(int V, int nx, int ny_, int nz)
+        : per((unsigned)(nx / V)), ny((unsigned)ny_), all(per * ny * (unsigned)nz), by_per(per), by_ny(ny)
+    {
+    }
+};
+
 // f(dose, target) for every resin voxel (target only when given).  Threads take groups of V voxels,
 // kDeep of them in flight each.
 template <int V, bool kTarget, typename DT, typename F>
 __device__ __forceinline__ void each_resin(const DT *__restrict__ dose, const float *__restrict__ target,
-                                           const int2 *__restrict__ span, int nx, int ny, int nz, F &&f)
+                                           const int2 *__restrict__ span, const Groups &G, F &&f)
 {
     constexpr int kDeep = kTarget ? 1 : 2;
-    const unsigned per = (unsigned)(nx / V), rows = (unsigned)ny * nz, all = rows * per, stride = gridDim.x * kRowThreads;
-    const float inv_per = 1.0f / (float)per, inv_ny = 1.0f / (float)ny;
-    // i / n through a reciprocal, corrected by one either way
-    auto div = [](unsigned i, unsigned n, float inv) {
-        unsigned q = (unsigned)((float)i * inv);
-        if (q * n > i) --q;
-        else if (i - q * n >= n) ++q;
-        return q;
-    };
+    const unsigned per = G.per, all = G.all, nx = per * V, stride = gridDim.x * kRowThreads;
     for (unsigned i0 = blockIdx.x * kRowThreads + threadIdx.x; i0 < all; i0 += kDeep * stride) {
         Group<V, DT> d[kDeep];
         Group<V, float> t[kTarget ? kDeep : 1];
@@ -75,9 +79,9 @@ __device__ __forceinline__ void each_resin(const DT *__restrict__ dose, const fl
             const unsigned i = i0 + k * stride;
             lo[k] = hi[k] = 0;
             if (i < all) {
-                const unsigned r = div(i, per, inv_per), z = div(r, (unsigned)ny, inv_ny);
+                const unsigned r = G.by_per(i), z = G.by_ny(r);
                 const int x = (int)(i - r * per) * V;
-                const int2 sp = span[r - z * ny];
+                const int2 sp = span[r - z * G.ny];
                 lo[k] = max(sp.x - x, 0);
                 hi[k] = min(sp.y - x, V);
                 if (lo[k] < hi[k]) {
@@ -104,24 +108,23 @@ constexpr int kMaxBlocks = 4, kHistBlocks = 4;      // per SM (2 and 3: within 5
 
 template <int V, typename DT>
 __global__ void __launch_bounds__(kRowThreads, kMaxBlocks)
-    dose_max_kernel(const DT *__restrict__ dose, const int2 *__restrict__ span, int nx, int ny, int nz,
-                    float *__restrict__ out)
+    dose_max_kernel(const DT *__restrict__ dose, const int2 *__restrict__ span, const Groups G, float *__restrict__ out)
 {
     float m = 0.f;
-    each_resin<V, false>(dose, nullptr, span, nx, ny, nz, [&](float d, float) { m = fmaxf(m, d); });
+    each_resin<V, false>(dose, nullptr, span, G, [&](float d, float) { m = fmaxf(m, d); });
     block_max(m, out);
 }
 
 template <int V, typename DT>
 __global__ void __launch_bounds__(kRowThreads, kHistBlocks)
-    ver_hist_kernel(const DT *__restrict__ dose, const float *__restrict__ target, const int2 *__restrict__ span, int nx,
-                    int ny, int nz, VerState *__restrict__ st, long long *__restrict__ out)
+    ver_hist_kernel(const DT *__restrict__ dose, const float *__restrict__ target, const int2 *__restrict__ span,
+                    const Groups G, VerState *__restrict__ st, long long *__restrict__ out)
 {
     __shared__ unsigned sh[2 * kBins];
     hist_clear(sh);
     __syncthreads();
     const float scale = hist_scale(st->dmax);
-    each_resin<V, true>(dose, target, span, nx, ny, nz, [&](float d, float t) { hist_add(sh, d, scale, t > 0.5f); });
+    each_resin<V, true>(dose, target, span, G, [&](float d, float t) { hist_add(sh, d, scale, t > 0.5f); });
     __syncthreads();
     hist_flush(sh, st->hist);
     if (last_block(&st->counter)) ver_scan(st->hist, out);
@@ -152,18 +155,18 @@ cudaError_t ver_t(const vamrt_projector *p, const DT *dose, const float *target,
     if (e != cudaSuccess) return e;
     constexpr int V = 16 / (int)sizeof(DT);
     const bool wide = nx % V == 0 && (((uintptr_t)dose | (uintptr_t)target) & 15) == 0;
-    const int64_t n = (int64_t)ny * nz * (wide ? nx / V : nx);
+    const Groups G(wide ? V : 1, nx, ny, nz);
     auto blocks = [&](int per_sm) {
-        const int64_t want = (n + kRowThreads - 1) / kRowThreads, cap = (int64_t)p->num_sms * per_sm;
+        const int64_t want = ((int64_t)G.all + kRowThreads - 1) / kRowThreads, cap = (int64_t)p->num_sms * per_sm;
         return (unsigned)(want < cap ? want : cap);
     };
     const unsigned gm = blocks(kMaxBlocks), gh = blocks(kHistBlocks);
     if (wide) {
-        dose_max_kernel<V><<<gm, kRowThreads, 0, s>>>(dose, p->spans, nx, ny, nz, &st->dmax);
-        ver_hist_kernel<V><<<gh, kRowThreads, 0, s>>>(dose, target, p->spans, nx, ny, nz, st, out3);
+        dose_max_kernel<V><<<gm, kRowThreads, 0, s>>>(dose, p->spans, G, &st->dmax);
+        ver_hist_kernel<V><<<gh, kRowThreads, 0, s>>>(dose, target, p->spans, G, st, out3);
     } else {
-        dose_max_kernel<1><<<gm, kRowThreads, 0, s>>>(dose, p->spans, nx, ny, nz, &st->dmax);
-        ver_hist_kernel<1><<<gh, kRowThreads, 0, s>>>(dose, target, p->spans, nx, ny, nz, st, out3);
+        dose_max_kernel<1><<<gm, kRowThreads, 0, s>>>(dose, p->spans, G, &st->dmax);
+        ver_hist_kernel<1><<<gh, kRowThreads, 0, s>>>(dose, target, p->spans, G, st, out3);
     }
     count_launches(2);
     return cudaGetLastError();
