@@ -6,7 +6,8 @@
  * C ABI.  Every entry point takes plain pointers and sizes, returns a vamrt_status and
  * never lets an exception or exit() cross the boundary.  Device buffers are owned by
  * the caller unless stated otherwise; the library owns only a projector handle (its ray
- * table, angle table and one scratch volume) and small reduction buffers.
+ * table, angle table, one scratch volume and, where its operators take angles in groups, four
+ * rotated copies of it: vamrt_get_groups) and small reduction buffers.
  *
  * Conventions (shared by every call):
  *   - Volume layout [nz][ny][nx], x fastest; voxel (i,j,k) has its centre at
@@ -153,7 +154,7 @@ typedef struct {
     int64_t n_rays;            /* nu * nv * rays_per_pixel */
     int64_t rays_in_resin;     /* rays that reach the resin */
     uint64_t samples_per_pass; /* n_angles * sum over rays of samples reaching the grid */
-    uint64_t scratch_bytes;    /* device bytes owned by the handle (table + scratch) */
+    uint64_t scratch_bytes;    /* device bytes owned by the handle (table + scratch + rotated copies) */
 } vamrt_info;
 
 /*
@@ -173,6 +174,23 @@ void vamrt_destroy_projector(vamrt_projector *p);
 
 /* Sizes, ray counts and the exact number of ray-voxel samples one operator pass visits. */
 vamrt_status vamrt_get_info(const vamrt_projector *p, vamrt_info *info);
+
+/*
+ * How many angles the handle's operators walk together, written to out[2] (host array): out[0] for
+ * vamrt_adjoint, out[1] for vamrt_forward_dose (4: a quarter turn apart, 2: half a turn, 1: one at a
+ * time).  Groups need four rotated FP32 copies of the volume, which vamrt_make_projector allocates
+ * only where at least as much device memory stays free; without them every call works one
+ * angle at a time, with the same results to rounding.  Error: EINVAL (NULL).
+ */
+vamrt_status vamrt_get_groups(const vamrt_projector *p, int32_t *out);
+
+/*
+ * The same for a geometry, before a projector is made: out[3] (host array) = {out[0], out[1] of
+ * vamrt_get_groups, bytes of the copies and their tables (0 without groups)} on a device of `sms`
+ * SMs with free_bytes of memory free.  Host-only, launches nothing.  Errors: EINVAL (NULL, sms < 1,
+ * bad geometry), ENOMEM.
+ */
+vamrt_status vamrt_group_plan(const vamrt_geometry *geom, int32_t sms, uint64_t free_bytes, int64_t *out);
 
 /* Samples per pass (same as vamrt_get_info's samples_per_pass). */
 vamrt_status vamrt_sample_count(const vamrt_projector *p, uint64_t *samples_per_pass);

@@ -115,7 +115,7 @@ struct vamrt_projector {
     vamrt::OpParams op;
     int ring_s;                // angles per group of the grouped projection; 0: not set up
     int ring_dose;             // the dose is grouped too
-    float *ring_vols;          // 4 rotated copies of the volume, or dose accumulators
+    float *ring_vols;          // 4 rotated copies of the volume, or dose accumulators; the others lie behind them
     unsigned char *ring_bricks;
     double2 *ring_cs;
     int *ring_members;
@@ -156,6 +156,7 @@ cudaError_t launch_unpad_acc(const vamrt_projector *p, const float *acc, void *d
 // maps of the rotated copies, and the launches: spread = caller's volume -> rotated copies.
 int plan_ring_groups(const double *theta, int n, int max_s, std::vector<int> &members, std::vector<double> &base);
 int ring_ex_classes(int S);
+size_t ring_map_count(int S);
 cudaError_t ring_maps(const RingParams &G, int S, const float *vols, std::vector<CUtensorMap> &maps);
 cudaError_t launch_ring_spread(const vamrt_projector *p, const void *vol, vamrt_dtype dt, cudaStream_t s);
 cudaError_t launch_ring_project(const vamrt_projector *p, void *proj, vamrt_dtype dt, uint32_t flags, cudaStream_t s);

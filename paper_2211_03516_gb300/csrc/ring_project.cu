@@ -425,6 +425,7 @@ int plan_ring_groups(const double *theta, int n, int max_s, std::vector<int> &me
 }
 
 int ring_ex_classes(int S) { return (kMaxEX - kMinEX) / (4 / S) + 1; }
+size_t ring_map_count(int S) { return (size_t)(4 / S) * ring_ex_classes(S) * (kMaxEZ / kStepEZ); }
 
 // Tensor maps of the rotated volumes for every window class, in the kernel's order.
 cudaError_t ring_maps(const RingParams &G, int S, const float *vols, std::vector<CUtensorMap> &maps)
@@ -432,7 +433,7 @@ cudaError_t ring_maps(const RingParams &G, int S, const float *vols, std::vector
     PFN_cuTensorMapEncodeTiled_v12000 enc = tma_encoder();
     if (!enc) return cudaErrorNotSupported;
     const int exq = 4 / S, n_ex = ring_ex_classes(S), n_ez = kMaxEZ / kStepEZ;
-    maps.resize((size_t)(4 / S) * n_ex * n_ez);
+    maps.resize(ring_map_count(S));
     for (int w = 0; w < 4 / S; ++w) {
         const int odd = S == 4 ? 0 : (w & 1);
         const cuuint64_t ex = (cuuint64_t)(odd ? G.op.ny : G.op.nx) + 2, ey = (cuuint64_t)(odd ? G.op.nx : G.op.ny) + 2;

@@ -159,10 +159,6 @@ void release(vamrt_projector *p)
     cudaFree(p->ver);
     cudaFree(p->spans);
     cudaFree(p->ring_vols);
-    cudaFree(p->ring_bricks);
-    cudaFree(p->ring_cs);
-    cudaFree(p->ring_members);
-    cudaFree(p->ring_maps);
     if (p->host_err) cudaFreeHost(p->host_err);
     if (cur >= 0 && cur != p->device) cudaSetDevice(cur);
     delete p;
@@ -179,62 +175,111 @@ struct Guard {
 //   grouped 40 us, per angle 37; 36 angles, 576 blocks: 41 against 61).
 //   Dose: more than three (54 x 54 x 76, 4 rays, 48 angles, 1296 blocks: 264 against 212 us;
 //   128^3, 24 angles, 1536 blocks: 643 against 716).
-bool grouped_projection_pays(const vamrt_projector *p, int64_t blocks) { return blocks > 3 * (int64_t)p->num_sms; }
-bool grouped_dose_pays(const vamrt_projector *p, int64_t blocks) { return blocks > 9 * (int64_t)p->num_sms; }
+bool grouped_projection_pays(int sms, int64_t blocks) { return blocks > 3 * (int64_t)sms; }
+bool grouped_dose_pays(int sms, int64_t blocks) { return blocks > 9 * (int64_t)sms; }
 
-// The grouped operators' groups, rotated copies and tensor maps (ring.cuh).  Scans without
-// partner angles, small scans, handles that cannot have four times the scratch volume, and
-// grids longer than the kernels' window arithmetic and launch grids reach keep the per-angle
-// operators.
+// The scan's angles, FP64
+std::vector<double> scan_angles(const vamrt_geometry &g)
+{
+    std::vector<double> theta((size_t)g.n_angles);
+    for (int k = 0; k < g.n_angles; ++k) theta[(size_t)k] = g.angles_rad ? g.angles_rad[k] : 2.0 * M_PI * k / g.n_angles;
+    return theta;
+}
+
+// The grouped operators' groups and the one device allocation that holds what they need (ring.cuh):
+// four rotated copies of the volume, then bricks, groups and tensor maps.
+struct GroupPlan {
+    int S = 0;                     // angles per group of the projection; 0: one at a time
+    bool dose = false;             // the dose is grouped too
+    int pzp = 0, bzp = 0;
+    int64_t vol_elems = 0, brick_stride = 0;
+    std::vector<int> members;
+    std::vector<double> base;
+    uint64_t bricks = 0, cs = 0, list = 0, maps = 0, bytes = 0;     // offsets, size
+};
+
+// Scans without partner angles, small scans, and grids longer than the kernels' window arithmetic and
+// launch grids reach keep the per-angle operators (S = 0).  Host only; may throw bad_alloc.
+GroupPlan plan_groups(const vamrt_geometry &g, const std::vector<double> &theta, int sms)
+{
+    GroupPlan pl;
+    const int64_t blocks = (int64_t)((g.nu + 7) / 8) * ((g.nv + 31) / 32) * g.n_angles;
+    if (!grouped_projection_pays(sms, blocks) || g.nx > 8192 || g.ny > 8192 || g.nz > 8192) return pl;
+    pl.pzp = (g.nz + 2 + 3) & ~3;
+    pl.vol_elems = (int64_t)(g.nx + 2) * (g.ny + 2) * pl.pzp;
+    if (pl.vol_elems >= (int64_t)1 << 31) return pl;
+    pl.S = vamrt::plan_ring_groups(theta.data(), (int)theta.size(), g.nx == g.ny ? 4 : 2, pl.members, pl.base);
+    if (pl.S == 0) return pl;                           // no partners
+    pl.dose = pl.S == 4 && grouped_dose_pays(sms, blocks);
+    pl.bzp = ((pl.pzp + 7) / 8 + 7) & ~7;
+    pl.brick_stride = (int64_t)((g.nx + 2 + 7) / 8) * ((g.ny + 2 + 7) / 8) * pl.bzp;
+    auto place = [&](uint64_t bytes) {
+        const uint64_t at = pl.bytes;
+        pl.bytes = (at + bytes + 255) & ~(uint64_t)255;
+        return at;
+    };
+    place(sizeof(float) * 4 * (uint64_t)pl.vol_elems);
+    pl.bricks = place((uint64_t)(4 / pl.S) * pl.brick_stride);
+    pl.cs = place(sizeof(double2) * pl.base.size());
+    pl.list = place(sizeof(int) * pl.members.size());
+    pl.maps = place(sizeof(CUtensorMap) * vamrt::ring_map_count(pl.S));
+    return pl;
+}
+
+// The copies are taken only where at least as much memory stays free: a caller's volumes and
+// projections, often made after the handle, come first.
+bool copies_fit(uint64_t bytes, uint64_t free_bytes) { return bytes <= free_bytes / 2; }
+
+// Sets the grouped operators up where they pay and their memory can be had; the handle keeps the
+// per-angle operators otherwise.
 vamrt_status setup_ring(vamrt_projector *p, const std::vector<double> &theta, cudaStream_t s)
 {
     const vamrt_geometry &g = p->g;
     p->ring_s = 0;
     p->ring_dose = 0;
-    const int64_t blocks = (int64_t)((g.nu + 7) / 8) * ((g.nv + 31) / 32) * g.n_angles;
-    if (!grouped_projection_pays(p, blocks) || g.nx > 8192 || g.ny > 8192 || g.nz > 8192) return VAMRT_OK;
-    vamrt::RingParams &G = p->ring;
-    G.op = p->op;
-    G.pzp = (g.nz + 2 + 3) & ~3;
-    G.vol_elems = (int64_t)(g.nx + 2) * (g.ny + 2) * G.pzp;
-    if (G.vol_elems >= (int64_t)1 << 31) return VAMRT_OK;
-    std::vector<int> members;
+    GroupPlan pl;
     std::vector<double2> cs;
-    std::vector<CUtensorMap> maps;
-    int S = 0;
     try {
-        std::vector<double> base;
-        S = vamrt::plan_ring_groups(theta.data(), (int)theta.size(), g.nx == g.ny ? 4 : 2, members, base);
-        for (double th : base) cs.push_back(make_double2(cos(th), sin(th)));
+        pl = plan_groups(g, theta, p->num_sms);
+        for (double th : pl.base) cs.push_back(make_double2(cos(th), sin(th)));
     } catch (...) {
         return fail(VAMRT_ENOMEM, "host allocation failed");
     }
-    if (S == 0) return VAMRT_OK;                        // no partners
-    if (cudaMalloc(&p->ring_vols, sizeof(float) * 4 * (size_t)G.vol_elems) != cudaSuccess) {
+    if (pl.S == 0) return VAMRT_OK;
+    size_t free_bytes = 0, total = 0;
+    CK(cudaMemGetInfo(&free_bytes, &total), "cudaMemGetInfo");
+    if (!copies_fit(pl.bytes, free_bytes)) return VAMRT_OK;
+    if (cudaMalloc(&p->ring_vols, (size_t)pl.bytes) != cudaSuccess) {
         cudaGetLastError();
         p->ring_vols = nullptr;
         return VAMRT_OK;
     }
+    char *const base = reinterpret_cast<char *>(p->ring_vols);
+    p->ring_bricks = reinterpret_cast<unsigned char *>(base + pl.bricks);
+    p->ring_cs = reinterpret_cast<double2 *>(base + pl.cs);
+    p->ring_members = reinterpret_cast<int *>(base + pl.list);
+    p->ring_maps = reinterpret_cast<CUtensorMap *>(base + pl.maps);
+    vamrt::RingParams &G = p->ring;
+    G.op = p->op;
+    G.pzp = pl.pzp;
+    G.vol_elems = pl.vol_elems;
+    G.bzp = pl.bzp;
+    G.brick_stride = pl.brick_stride;
+    std::vector<CUtensorMap> maps;
     cudaError_t e = cudaSuccess;
     try {
-        e = vamrt::ring_maps(G, S, p->ring_vols, maps);
+        e = vamrt::ring_maps(G, pl.S, p->ring_vols, maps);
     } catch (...) {
         return fail(VAMRT_ENOMEM, "host allocation failed");
     }
-    if (e == cudaErrorNotSupported) {                   // no tensor-map encoder
+    if (e != cudaSuccess) {                             // no tensor-map encoder, or one that refuses the copies
         cudaFree(p->ring_vols);
         p->ring_vols = nullptr;
         return VAMRT_OK;
     }
-    if (e != cudaSuccess) return cuda_fail(e, "tensor maps");
-    G.bzp = ((G.pzp + 7) / 8 + 7) & ~7;
-    G.brick_stride = (int64_t)((g.nx + 2 + 7) / 8) * ((g.ny + 2 + 7) / 8) * G.bzp;
-    CK(cudaMalloc(&p->ring_bricks, (size_t)(4 / S) * G.brick_stride), "cudaMalloc(bricks)");
-    CK(cudaMalloc(&p->ring_cs, sizeof(double2) * cs.size()), "cudaMalloc(groups)");
-    CK(cudaMalloc(&p->ring_members, sizeof(int) * members.size()), "cudaMalloc(groups)");
-    CK(cudaMalloc(&p->ring_maps, sizeof(CUtensorMap) * maps.size()), "cudaMalloc(tensor maps)");
     CK(cudaMemcpyAsync(p->ring_cs, cs.data(), sizeof(double2) * cs.size(), cudaMemcpyHostToDevice, s), "copy");
-    CK(cudaMemcpyAsync(p->ring_members, members.data(), sizeof(int) * members.size(), cudaMemcpyHostToDevice, s), "copy");
+    CK(cudaMemcpyAsync(p->ring_members, pl.members.data(), sizeof(int) * pl.members.size(), cudaMemcpyHostToDevice, s),
+       "copy");
     CK(cudaMemcpyAsync(p->ring_maps, maps.data(), sizeof(CUtensorMap) * maps.size(), cudaMemcpyHostToDevice, s), "copy");
     CK(cudaStreamSynchronize(s), "sync");
     G.n_groups = (int)cs.size();
@@ -242,16 +287,15 @@ vamrt_status setup_ring(vamrt_projector *p, const std::vector<double> &theta, cu
     G.members = p->ring_members;
     G.bricks = p->ring_bricks;
     G.maps = p->ring_maps;
-    G.n_ex = vamrt::ring_ex_classes(S);
+    G.n_ex = vamrt::ring_ex_classes(pl.S);
     // Fixed-point units of the largest weight: a voxel's sum over a block's 256 rays stays
     // below 2^31, and one share -- up to the floor(2 sqrt(3) / step) + 1 samples of a ray in
     // one cell -- below the 2^22 that its conversion holds.
     const double run = floor(2.0 * sqrt(3.0) / g.step_vox) + 1.0;
     G.share_scale = (float)fmin(2147483648.0 / (1.01 * 256.0 * p->op.cell_bound), 4.1e6 / run);
-    p->device_bytes += sizeof(float) * 4 * (uint64_t)G.vol_elems + (uint64_t)(4 / S) * G.brick_stride + (sizeof(double2) + sizeof(int) * S) * (uint64_t)cs.size() +
-                       sizeof(CUtensorMap) * (uint64_t)maps.size();
-    p->ring_s = S;
-    p->ring_dose = S == 4 && grouped_dose_pays(p, blocks) ? 1 : 0;
+    p->device_bytes += pl.bytes;
+    p->ring_s = pl.S;
+    p->ring_dose = pl.dose ? 1 : 0;
     return VAMRT_OK;
 }
 
@@ -370,15 +414,12 @@ vamrt_status vamrt_make_projector(const vamrt_geometry *geom, void *stream, vamr
     std::vector<double> theta;
     std::vector<double2> hcs;
     try {
-        theta.resize((size_t)g.n_angles);
+        theta = scan_angles(*geom);
         hcs.resize((size_t)g.n_angles);
     } catch (...) {
         return fail(VAMRT_ENOMEM, "host allocation failed");
     }
-    for (int k = 0; k < g.n_angles; ++k) {
-        theta[(size_t)k] = geom->angles_rad ? geom->angles_rad[k] : 2.0 * M_PI * k / g.n_angles;
-        hcs[(size_t)k] = make_double2(cos(theta[(size_t)k]), sin(theta[(size_t)k]));
-    }
+    for (int k = 0; k < g.n_angles; ++k) hcs[(size_t)k] = make_double2(cos(theta[(size_t)k]), sin(theta[(size_t)k]));
     cudaError_t e = cudaMemcpyAsync(p->cs, hcs.data(), sizeof(double2) * g.n_angles, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return cuda_fail(e, "angle table upload");
@@ -465,6 +506,31 @@ vamrt_status vamrt_get_info(const vamrt_projector *p, vamrt_info *info)
     info->rays_in_resin = p->rays_in_resin;
     info->samples_per_pass = p->samples_per_angle * (uint64_t)p->g.n_angles;
     info->scratch_bytes = p->device_bytes;
+    return VAMRT_OK;
+}
+
+vamrt_status vamrt_group_plan(const vamrt_geometry *geom, int32_t sms, uint64_t free_bytes, int64_t *out)
+{
+    if (!out || sms < 1) return fail(VAMRT_EINVAL, "NULL out or sms < 1");
+    const vamrt_status st = validate(geom);
+    if (st != VAMRT_OK) return st;
+    try {
+        const GroupPlan pl = plan_groups(*geom, scan_angles(*geom), sms);
+        const bool on = pl.S != 0 && copies_fit(pl.bytes, free_bytes);
+        out[0] = on ? pl.S : 1;
+        out[1] = on && pl.dose ? pl.S : 1;
+        out[2] = on ? (int64_t)pl.bytes : 0;
+    } catch (...) {
+        return fail(VAMRT_ENOMEM, "host allocation failed");
+    }
+    return VAMRT_OK;
+}
+
+vamrt_status vamrt_get_groups(const vamrt_projector *p, int32_t *out)
+{
+    if (!p || !out) return fail(VAMRT_EINVAL, "NULL argument");
+    out[0] = p->ring_s ? p->ring_s : 1;
+    out[1] = p->ring_dose ? p->ring_s : 1;
     return VAMRT_OK;
 }
 

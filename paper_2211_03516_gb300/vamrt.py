@@ -94,6 +94,10 @@ def lib() -> ctypes.CDLL:
         L.vamrt_destroy_projector.restype = None
         L.vamrt_get_info.argtypes = [vp, ctypes.POINTER(Info)]
         L.vamrt_sample_count.argtypes = [vp, ctypes.POINTER(ctypes.c_uint64)]
+        L.vamrt_get_groups.argtypes = [vp, ctypes.POINTER(ctypes.c_int32)]
+        L.vamrt_get_groups.restype = i32
+        L.vamrt_group_plan.argtypes = [ctypes.POINTER(Geometry), i32, ctypes.c_uint64, ctypes.POINTER(ctypes.c_int64)]
+        L.vamrt_group_plan.restype = i32
         L.vamrt_adjoint.argtypes = [vp, vp, i32, vp, i32, u32, vp]
         L.vamrt_forward_dose.argtypes = [vp, vp, i32, vp, i32, u32, vp]
         L.vamrt_optimize.argtypes = [vp, vp, vp, vp, vp, ctypes.POINTER(OptParams), ctypes.POINTER(OptReport), vp]
@@ -236,6 +240,16 @@ def vamrt_make_projector(spec: GeometrySpec, stream=None) -> ctypes.c_void_p:
     return h
 
 
+def group_plan(spec: GeometrySpec, sms: int, free_bytes: int):
+    """(angles walked together by adjoint, by forward_dose, bytes of the copies that needs)
+    (vamrt_group_plan)."""
+    g, keep = _to_struct(spec)
+    out = (ctypes.c_int64 * 3)()
+    _check(lib().vamrt_group_plan(ctypes.byref(g), sms, free_bytes, out), "vamrt_group_plan")
+    del keep
+    return tuple(out)
+
+
 class Projector:
     """Owns one vamrt_projector handle.  Operators run on the current torch stream."""
 
@@ -265,6 +279,12 @@ class Projector:
         _check(lib().vamrt_get_info(self.handle, ctypes.byref(i)), "vamrt_get_info")
         return dict(n_rays=i.n_rays, rays_in_resin=i.rays_in_resin, samples_per_pass=i.samples_per_pass,
                     scratch_bytes=i.scratch_bytes)
+
+    def groups(self):
+        """(angles walked together by adjoint, by forward_dose); 1: one at a time (vamrt_get_groups)."""
+        out = (ctypes.c_int32 * 2)()
+        _check(lib().vamrt_get_groups(self.handle, out), "vamrt_get_groups")
+        return tuple(out)
 
     def sample_count(self) -> int:
         n = ctypes.c_uint64()
