@@ -187,10 +187,12 @@ vamrt_status vamrt_get_groups(const vamrt_projector *p, int32_t *out);
 /*
  * The same for a geometry, before a projector is made: out[3] (host array) = {out[0], out[1] of
  * vamrt_get_groups, bytes of the copies and their tables (0 without groups)} on a device of `sms`
- * SMs with free_bytes of memory free.  Host-only, launches nothing.  Errors: EINVAL (NULL, sms < 1,
- * bad geometry), ENOMEM.
+ * SMs with free_bytes of memory free, for a pass of `samples` samples (vamrt_sample_count; few for
+ * the volume's size do not pay for its copies).  Host-only, launches nothing.  Errors: EINVAL (NULL,
+ * sms < 1, bad geometry), ENOMEM.
  */
-vamrt_status vamrt_group_plan(const vamrt_geometry *geom, int32_t sms, uint64_t free_bytes, int64_t *out);
+vamrt_status vamrt_group_plan(const vamrt_geometry *geom, int32_t sms, uint64_t samples, uint64_t free_bytes,
+                              int64_t *out);
 
 /* Samples per pass (same as vamrt_get_info's samples_per_pass). */
 vamrt_status vamrt_sample_count(const vamrt_projector *p, uint64_t *samples_per_pass);

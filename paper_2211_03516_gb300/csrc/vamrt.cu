@@ -178,6 +178,13 @@ struct Guard {
 bool grouped_projection_pays(int sms, int64_t blocks) { return blocks > 3 * (int64_t)sms; }
 bool grouped_dose_pays(int sms, int64_t blocks) { return blocks > 9 * (int64_t)sms; }
 
+// Whether a pass visits enough samples for what four copies of the volume cost to write, or to clear
+// and gather.  Dose and projection of volumes without a zero, us, grouped against per angle, 768 x 768 x 1024
+// and chief rays: groups of four 5394 / 4780 against 4273 / 2287 at 0.9 samples per voxel, 7857 / 6180 against
+// 8672 / 6043 at 4.2, 10310 / 7631 against 12980 / 9754 at 7.4; groups of two (projection) 11062 against 9862
+// at 7.5, 16027 against 18391 at 14.9; 384 x 384 x 512: 1330 against 1298 at 7.4, 1958 against 2352 at 14.7.
+bool copies_pay(int S, double samples, double voxels) { return samples > (S == 4 ? 5.0 : 10.0) * voxels; }
+
 // The scan's angles, FP64
 std::vector<double> scan_angles(const vamrt_geometry &g)
 {
@@ -198,9 +205,10 @@ struct GroupPlan {
     uint64_t bricks = 0, cs = 0, list = 0, maps = 0, bytes = 0;     // offsets, size
 };
 
-// Scans without partner angles, small scans, and grids longer than the kernels' window arithmetic and
-// launch grids reach keep the per-angle operators (S = 0).  Host only; may throw bad_alloc.
-GroupPlan plan_groups(const vamrt_geometry &g, const std::vector<double> &theta, int sms)
+// Scans without partner angles, small scans, scans of few samples (of a pass) for their volume, and grids
+// longer than the kernels' window arithmetic and launch grids reach keep the per-angle operators (S
+// = 0).  Host only; may throw bad_alloc.
+GroupPlan plan_groups(const vamrt_geometry &g, const std::vector<double> &theta, int sms, uint64_t samples)
 {
     GroupPlan pl;
     const int64_t blocks = (int64_t)((g.nu + 7) / 8) * ((g.nv + 31) / 32) * g.n_angles;
@@ -209,7 +217,8 @@ GroupPlan plan_groups(const vamrt_geometry &g, const std::vector<double> &theta,
     pl.vol_elems = (int64_t)(g.nx + 2) * (g.ny + 2) * pl.pzp;
     if (pl.vol_elems >= (int64_t)1 << 31) return pl;
     pl.S = vamrt::plan_ring_groups(theta.data(), (int)theta.size(), g.nx == g.ny ? 4 : 2, pl.members, pl.base);
-    if (pl.S == 0) return pl;                           // no partners
+    if (pl.S != 0 && !copies_pay(pl.S, (double)samples, (double)g.nx * g.ny * g.nz)) pl.S = 0;
+    if (pl.S == 0) return pl;
     pl.dose = pl.S == 4 && grouped_dose_pays(sms, blocks);
     pl.bzp = ((pl.pzp + 7) / 8 + 7) & ~7;
     pl.brick_stride = (int64_t)((g.nx + 2 + 7) / 8) * ((g.ny + 2 + 7) / 8) * pl.bzp;
@@ -240,7 +249,7 @@ vamrt_status setup_ring(vamrt_projector *p, const std::vector<double> &theta, cu
     GroupPlan pl;
     std::vector<double2> cs;
     try {
-        pl = plan_groups(g, theta, p->num_sms);
+        pl = plan_groups(g, theta, p->num_sms, p->samples_per_angle * (uint64_t)g.n_angles);
         for (double th : pl.base) cs.push_back(make_double2(cos(th), sin(th)));
     } catch (...) {
         return fail(VAMRT_ENOMEM, "host allocation failed");
@@ -509,13 +518,14 @@ vamrt_status vamrt_get_info(const vamrt_projector *p, vamrt_info *info)
     return VAMRT_OK;
 }
 
-vamrt_status vamrt_group_plan(const vamrt_geometry *geom, int32_t sms, uint64_t free_bytes, int64_t *out)
+vamrt_status vamrt_group_plan(const vamrt_geometry *geom, int32_t sms, uint64_t samples, uint64_t free_bytes,
+                              int64_t *out)
 {
     if (!out || sms < 1) return fail(VAMRT_EINVAL, "NULL out or sms < 1");
     const vamrt_status st = validate(geom);
     if (st != VAMRT_OK) return st;
     try {
-        const GroupPlan pl = plan_groups(*geom, scan_angles(*geom), sms);
+        const GroupPlan pl = plan_groups(*geom, scan_angles(*geom), sms, samples);
         const bool on = pl.S != 0 && copies_fit(pl.bytes, free_bytes);
         out[0] = on ? pl.S : 1;
         out[1] = on && pl.dose ? pl.S : 1;

@@ -96,7 +96,8 @@ def lib() -> ctypes.CDLL:
         L.vamrt_sample_count.argtypes = [vp, ctypes.POINTER(ctypes.c_uint64)]
         L.vamrt_get_groups.argtypes = [vp, ctypes.POINTER(ctypes.c_int32)]
         L.vamrt_get_groups.restype = i32
-        L.vamrt_group_plan.argtypes = [ctypes.POINTER(Geometry), i32, ctypes.c_uint64, ctypes.POINTER(ctypes.c_int64)]
+        L.vamrt_group_plan.argtypes = [ctypes.POINTER(Geometry), i32, ctypes.c_uint64, ctypes.c_uint64,
+                                       ctypes.POINTER(ctypes.c_int64)]
         L.vamrt_group_plan.restype = i32
         L.vamrt_adjoint.argtypes = [vp, vp, i32, vp, i32, u32, vp]
         L.vamrt_forward_dose.argtypes = [vp, vp, i32, vp, i32, u32, vp]
@@ -240,12 +241,12 @@ def vamrt_make_projector(spec: GeometrySpec, stream=None) -> ctypes.c_void_p:
     return h
 
 
-def group_plan(spec: GeometrySpec, sms: int, free_bytes: int):
+def group_plan(spec: GeometrySpec, sms: int, samples: int, free_bytes: int):
     """(angles walked together by adjoint, by forward_dose, bytes of the copies that needs)
     (vamrt_group_plan)."""
     g, keep = _to_struct(spec)
     out = (ctypes.c_int64 * 3)()
-    _check(lib().vamrt_group_plan(ctypes.byref(g), sms, free_bytes, out), "vamrt_group_plan")
+    _check(lib().vamrt_group_plan(ctypes.byref(g), sms, samples, free_bytes, out), "vamrt_group_plan")
     del keep
     return tuple(out)
 

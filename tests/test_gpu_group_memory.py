@@ -20,13 +20,13 @@ def V():
 
 def test_a_handle_made_while_memory_is_short(V):
     """It works one angle at a time, with the same results; one made with memory to spare groups."""
-    w = I.TINY.scaled(nx=480, ny=480, nz=600, voxel_mm=0.05, nu=64, nv=64, pixel_u_mm=0.3, pixel_v_mm=0.4, r_inner_mm=11.8,
+    w = I.TINY.scaled(nx=480, ny=480, nz=600, voxel_mm=0.05, nu=96, nv=96, pixel_u_mm=0.2, pixel_v_mm=0.27, r_inner_mm=11.8,
                       n_angles=180)
     pupil = I.workload_pupil(w)
     gen = torch.Generator(device="cuda:0").manual_seed(55)
     f = torch.rand(w.vol_shape, device="cuda:0", generator=gen)
-    bytes_ = V.group_plan(V.GeometrySpec.from_workload(w, pupil), 152, 1 << 40)[2]
-    y = torch.empty((180, 64, 64), device="cuda:0")
+    bytes_ = V.group_plan(V.GeometrySpec.from_workload(w, pupil), 152, 1 << 40, 1 << 40)[2]
+    y = torch.empty((180, 96, 96), device="cuda:0")
     d = torch.empty(w.vol_shape, device="cuda:0")
     torch.cuda.synchronize()
     torch.cuda.empty_cache()

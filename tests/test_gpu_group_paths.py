@@ -34,6 +34,16 @@ def test_every_scan_takes_its_path(V):
         assert V.Projector.from_workload(w, I.workload_pupil(w), angles_rad=angles).groups() == PATHS[name], name
 
 
+@pytest.mark.parametrize("nu,n_angles,want", [(32, 720, (4, 4)), (16, 480, (1, 1)), (32, 722, (2, 1)), (16, 722, (1, 1))])
+def test_small_pixel_arrays_over_a_large_grid(V, nu, n_angles, want):
+    """About 22, 3.6, 22 and 5.5 samples per voxel: below 5 (groups of four) or 10 (of two) the copies of the
+    volume cost more than groups save."""
+    w = I.TINY.scaled(nx=256, ny=256, nz=256, voxel_mm=0.1, nu=nu, nv=nu, pixel_u_mm=0.4, pixel_v_mm=0.4, r_inner_mm=12.5,
+                      n_angles=n_angles)
+    P = V.Projector.from_workload(w, I.workload_pupil(w))
+    assert P.groups() == want, P.sample_count() / 256 ** 3
+
+
 def test_a_scan_above_the_limits(V):
     pupil = I.workload_pupil(MANY)
     P = V.Projector.from_workload(MANY, pupil)

@@ -1,5 +1,6 @@
 """Which scans the operators take in groups of angles, by the host-only query (no GPU): partners,
-sizes on both sides of the limits, and the memory that the rotated copies may take."""
+sizes on both sides of the limits, samples for the volume's size, and the memory that the rotated
+copies may take."""
 import pytest
 
 from paper_2211_03516_gb300 import inputs as I
@@ -9,11 +10,11 @@ BASE = I.TINY.scaled(nx=35, ny=35, nz=41, voxel_mm=0.36, nu=37, nv=43, pixel_u_m
                      f_number=3.5, pupil_pattern="sunflower", rays_per_pixel=2, pupil_mm=60.0)     # 10 pixel tiles
 
 
-def _plan(w, sms=152, free=PLENTY, angles=None):
+def _plan(w, sms=152, free=PLENTY, angles=None, samples=PLENTY):
     from paper_2211_03516_gb300 import build
     build.build()
     from paper_2211_03516_gb300 import vamrt
-    return vamrt.group_plan(vamrt.GeometrySpec.from_workload(w, I.workload_pupil(w), angles), sms, free)
+    return vamrt.group_plan(vamrt.GeometrySpec.from_workload(w, I.workload_pupil(w), angles), sms, samples, free)
 
 
 @pytest.mark.parametrize("kw,want", [
@@ -33,6 +34,13 @@ def test_angle_lists():
     even = I.default_angles(144)
     assert _plan(BASE, angles=even[::-1] + 0.3)[:2] == (4, 4)
     assert _plan(BASE, angles=even ** 1.01)[:2] == (1, 1)
+
+
+def test_few_samples_for_the_volume():
+    voxels = 35 * 35 * 41
+    assert _plan(BASE, samples=5 * voxels)[:2] == (1, 1) and _plan(BASE, samples=5 * voxels + 1)[:2] == (4, 4)
+    half, voxels = BASE.scaled(ny=38), 35 * 38 * 41
+    assert _plan(half, samples=10 * voxels)[:2] == (1, 1) and _plan(half, samples=10 * voxels + 1)[:2] == (2, 1)
 
 
 def test_copies_leave_as_much_memory_free():
