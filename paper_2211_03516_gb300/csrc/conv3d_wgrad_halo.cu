@@ -33,9 +33,13 @@
 // 33, 48 -> 16 on 100 x 90 x 80 754 -> 57.  What bounds it now: an MMA of 128 x 48 x 16 takes 77
 // cycles, of which its operands' reads are most.
 //
-// A dY row or plane past the volume is zero, as are x < 0 and x >= W of the shifted copies: they
-// meet real X values there, so a voxel on a face of X that is not finite spoils all 27 taps of its
-// channel, as one inside does, and not only those that reach it from within the volume.
+// Values that are not finite.  Positions outside the volume meet real voxels of X (x = -1 and x = W of
+// the shifted copies of dY, rows and planes past the volume of a last tile): dY is zero there, but
+// its product with an X that is not finite is not, while a dY that is not finite does not meet the
+// zeros beside the volume in x.  Either leaves a sum of its row of M that is not finite, so the rows
+// that have one when TMEM is drained are summed again from global memory by the definition (direct_row).
+// Nothing else pays for it: 48 -> 16 channels on 184 x 128 x 128 264.0 -> 264.9 us (a warp that looks at every
+// tile's faces ahead of its MMAs: 317); with one infinite voxel 5.6 ms, x all NaN 17 ms.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <cuda_bf16.h>
@@ -61,7 +65,8 @@ struct Args {
     float *dW;
     int *err;
     WgradHaloPlan p;
-    int Cin;
+    int Cin, Cout, D, H, W;
+    const __nv_bfloat16 *X, *dY;
 };
 
 // box at channel 0 of slot (x, y) and the outer coordinates u, v
@@ -85,30 +90,97 @@ __device__ __forceinline__ TileRange tiles_of(const WgradHaloPlan &p, int b)
     return {(int)((int64_t)b * p.run * p.ntiles / p.npos), b == p.nsplit - 1 ? p.ntiles : (int)last, 1};
 }
 
-// Add accumulators tile0, tile0 + step, ... of this warp's 32 TMEM lanes into dW: lane 32 q + l is
-// row 16 s + ci of M, s = 8 tile + 2 q + l / 16
-__device__ __forceinline__ void drain(const Args &a, uint32_t tmem, int q, int lane, int tile0, int step, int chunk0,
-                                      int co0)
+__device__ __forceinline__ bool finite(float x) { return fabsf(x) <= 3.402823466e38f; }
+
+// By a warp, lane l for output channel co0 + l % 16: adds the sums of tap row (dz, dy), channel ci over the
+// positions of `tiles`, zero padding and no other, into dW.  Its lanes' halves take alternate rows; sums
+// that are all NaN end it.
+__device__ __noinline__ void direct_row(const Args &a, const TileRange &tiles, int dz, int dy, int ci, int co0, int lane)
+{
+    const WgradHaloPlan &p = a.p;
+    double total[3] = {0.0, 0.0, 0.0};
+    for (int tile = tiles.first; tile < tiles.end; tile += tiles.step) {
+        const int tx = tile % p.nx, r = tile / p.nx, ty = r % p.ny, tz = r / p.ny;
+        const int q0 = tx * p.XB, q1 = q0 + p.XB;             // columns of X
+        for (int row = lane >> 4; row < p.TZ * p.TY; row += 2) {
+            const int z = tz * p.TZ + row / p.TY, y = ty * p.TY + row % p.TY, zx = z + dz - 1, yx = y + dy - 1;
+            if (z >= a.D || y >= a.H) continue;
+            const bool in = zx >= 0 && zx < a.D && yx >= 0 && yx < a.H;
+            const __nv_bfloat16 *xr = a.X + ((int64_t)(in ? zx : z) * a.H + (in ? yx : y)) * a.W * a.Cin + ci;
+            const __nv_bfloat16 *gr = a.dY + ((int64_t)z * a.H + y) * a.W * a.Cout + co0 + (lane & 15);
+            auto x = [&](int q) { return in ? __bfloat162float(xr[(int64_t)q * a.Cin]) : 0.f; };
+            auto g = [&](int px) { return __bfloat162float(gr[(int64_t)px * a.Cout]); };
+            float sum[3] = {0.f, 0.f, 0.f};                    // of positions q + 1, q, q - 1
+            if (q0 == 0) {
+                sum[0] = g(1) * x(0) + g(0) * 0.f;
+                sum[1] = g(0) * x(0);
+            }
+            if (q1 == a.W) {
+                sum[1] += g(a.W - 1) * x(a.W - 1);
+                sum[2] += g(a.W - 2) * x(a.W - 1) + g(a.W - 1) * 0.f;
+            }
+            const int qa = max(q0, 1), qb = min(q1, a.W - 1);
+            float before = g(qa - 1), at = g(qa);
+#pragma unroll 8
+            for (int q = qa; q < qb; ++q) {
+                const float after = g(q + 1), v = x(q);
+                sum[0] = fmaf(after, v, sum[0]);
+                sum[1] = fmaf(at, v, sum[1]);
+                sum[2] = fmaf(before, v, sum[2]);
+                before = at;
+                at = after;
+            }
+#pragma unroll
+            for (int dx = 0; dx < 3; ++dx) total[dx] += sum[dx];
+        }
+        const int nan = isnan(total[0]) && isnan(total[1]) && isnan(total[2]);
+        if (__all_sync(0xffffffffu, __shfl_xor_sync(0xffffffffu, nan, 16) | nan)) break;
+    }
+#pragma unroll
+    for (int dx = 0; dx < 3; ++dx) {
+        const double s = total[dx] + __shfl_xor_sync(0xffffffffu, total[dx], 16);
+        if (lane < 16) atomicAdd(a.dW + ((int64_t)(co0 + lane) * 27 + dz * 9 + dy * 3 + dx) * a.Cin + ci, (float)s);
+    }
+}
+
+// Add accumulators tile0, tile0 + step, ... of this warp's 32 TMEM lanes, the sums of `tiles`, into dW: lane
+// 32 q + l is row 16 s + ci of M, s = 8 tile + 2 q + l / 16
+__device__ __forceinline__ void drain(const Args &a, const TileRange &tiles, uint32_t tmem, int q, int lane, int tile0,
+                                      int step, int chunk0, int co0)
 {
     const WgradHaloPlan &p = a.p;
     const int N = 3 * p.Ct, RY = p.TY + 2, ncg = min(p.cg, a.Cin / 16 - chunk0);
     for (int m = tile0; m < p.nt; m += step) {
         const int s = 8 * m + 2 * q + (lane >> 4), dy = s % RY, ch = s / RY % p.cg, dz = s / RY / p.cg;
         const bool use = dy < 3 && dz < 3 && ch < ncg;
-        float *dst = a.dW + (int64_t)(dz * 9 + dy * 3) * a.Cin + 16 * (chunk0 + ch) + (lane & 15);
-        for (int n0 = 0; n0 < N; n0 += 16) {
-            float sum[16];
-            tmem_ld16(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(m * N + n0), sum);
-            for (int part = 1; part < p.kp; ++part) {
-                float v[16];
-                tmem_ld16(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)((part * p.nt + m) * N + n0), v);
+        const int ci = 16 * (chunk0 + ch) + (lane & 15);
+        for (int co = 0; co < p.Ct; co += 16) {
+            float sum[3][16];
+            bool whole = true;
 #pragma unroll
-                for (int j = 0; j < 16; ++j) sum[j] += v[j];
+            for (int dx = 0; dx < 3; ++dx) {
+                const int n0 = dx * p.Ct + co;
+                tmem_ld16(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(m * N + n0), sum[dx]);
+                for (int part = 1; part < p.kp; ++part) {
+                    float v[16];
+                    tmem_ld16(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)((part * p.nt + m) * N + n0), v);
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) sum[dx][j] += v[j];
+                }
+#pragma unroll
+                for (int j = 0; j < 16; ++j) whole &= finite(sum[dx][j]);
             }
-            const int dx = n0 / p.Ct, co = co0 + n0 - dx * p.Ct;
-            if (use) {
+            if (use && whole) {
+                float *dst = a.dW + ((int64_t)(co0 + co) * 27 + dz * 9 + dy * 3) * a.Cin + ci;
 #pragma unroll
-                for (int j = 0; j < 16; ++j) atomicAdd(dst + ((int64_t)(co + j) * 27 + dx) * a.Cin, sum[j]);
+                for (int dx = 0; dx < 3; ++dx)
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) atomicAdd(dst + ((int64_t)j * 27 + dx) * a.Cin, sum[dx][j]);
+            }
+            for (unsigned again = __ballot_sync(0xffffffffu, use && !whole); again; again &= again - 1) {
+                const int l = __ffs(again) - 1;
+                direct_row(a, tiles, __shfl_sync(0xffffffffu, dz, l), __shfl_sync(0xffffffffu, dy, l),
+                           __shfl_sync(0xffffffffu, ci, l), co0 + co, lane);
             }
         }
     }
@@ -116,7 +188,7 @@ __device__ __forceinline__ void drain(const Args &a, uint32_t tmem, int q, int l
 
 __global__ void __launch_bounds__(kWgThreads, 1)
     conv3d_wgrad_halo_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUtensorMap ymap,
-                             const Args a)
+                             const __grid_constant__ Args a)
 {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     // full[slots], empty[slots], then: segment's MMAs done, segment drained, all MMAs done
@@ -196,7 +268,7 @@ __global__ void __launch_bounds__(kWgThreads, 1)
                     ok = mbar_wait(seg_done, k & 1);
                     if (__all_sync(0xffffffffu, ok)) {
                         tc_fence_after();
-                        drain(a, tmem, warp & 3, lane, 0, 1, chunk0, co0);
+                        drain(a, {tile - c * tiles.step, tile, tiles.step}, tmem, warp & 3, lane, 0, 1, chunk0, co0);
                         tc_fence_before();
                         __syncwarp();
                         if (lane == 0) mbar_arrive(drained);
@@ -247,7 +319,11 @@ __global__ void __launch_bounds__(kWgThreads, 1)
     }
     __syncthreads();
     tc_fence_after();
-    if (s_fin && !s_abort && tiles.first < tiles.end) drain(a, tmem, warp & 3, lane, warp >> 2, kWgThreads / 128, chunk0, co0);
+    if (s_fin && !s_abort && tiles.first < tiles.end) {
+        const int segs = ((tiles.end - tiles.first - 1) / tiles.step) / p.seg;        // added already
+        drain(a, {tiles.first + segs * p.seg * tiles.step, tiles.end, tiles.step}, tmem, warp & 3, lane, warp >> 2,
+              kWgThreads / 128, chunk0, co0);
+    }
     tc_fence_before();
     __syncthreads();
     if (warp == kIssuer0) tmem_dealloc(tmem, p.ncols);
@@ -351,7 +427,7 @@ cudaError_t launch_wgrad_halo(const void *X, const void *dY, float *dW, int D, i
     const int smem = std::max(pl.slots * pl.slot_bytes, 116 * 1024);
     cudaError_t e = cudaFuncSetAttribute(conv3d_wgrad_halo_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    const Args a{dW, err, pl, Cin};
+    const Args a{dW, err, pl, Cin, Cout, D, H, W, (const __nv_bfloat16 *)X, (const __nv_bfloat16 *)dY};
     conv3d_wgrad_halo_kernel<<<dim3(pl.ngroups * pl.nslices, pl.nsplit), kWgThreads, smem, s>>>(maps[0], maps[1], a);
     return cudaGetLastError();
 }
