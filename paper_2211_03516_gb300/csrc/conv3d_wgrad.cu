@@ -125,6 +125,9 @@ __global__ void __launch_bounds__(kTThreads, 2)
     const uint32_t tmem = s_tmem;
     const int s_begin = blockIdx.y * a.spb;
     const int n = max(0, min(a.spb, a.nstage - s_begin));
+    // K steps of a stage: none past the volume, where dy is zero but x may not be finite
+    const long long P = (long long)a.D * a.H * a.W;
+    auto ksteps = [&](int c) { return (int)min((long long)a.KS, P - (long long)(s_begin + c) * a.KS) / 16; };
 
     if (warp == 0) {
         // ---- producer: the stage's A boxes (plane it, box b) and B planes, spread over the lanes ----
@@ -165,7 +168,7 @@ __global__ void __launch_bounds__(kTThreads, 2)
     } else if (warp >= kTIssuer0 && warp - kTIssuer0 < nis) {
         // ---- issuers: accumulators k0, k0 + nis, ... = (tile acc / kp, K-step part acc % kp) ----
         if (lane == 0) {
-            const int k0 = warp - kTIssuer0, nks = a.KS / 16;
+            const int k0 = warp - kTIssuer0;
             const uint32_t idesc = instr_desc(128, a.Cout) | (1u << 15) | (1u << 16);   // A, B MN-major
             const uint64_t swA = (uint64_t)swizzle_layout(a.cwA) << 61, swB = (uint64_t)swizzle_layout(a.cwB) << 61;
             for (int c = 0; c < n; ++c) {
@@ -177,6 +180,7 @@ __global__ void __launch_bounds__(kTThreads, 2)
                 }
                 tc_fence_after();
                 const uint32_t sb = base + slot * a.slot_bytes;
+                const int nks = ksteps(c);
                 for (int acc = k0; acc < nacc; acc += nis) {
                     const int i = acc / a.kp, part = acc - i * a.kp;
                     for (int s = part; s < nks; s += a.kp)
@@ -199,13 +203,13 @@ __global__ void __launch_bounds__(kTThreads, 2)
     __syncthreads();
     tc_fence_after();
     if (s_fin && !s_abort && n > 0) {
-        const int q = warp & 3;
+        const int q = warp & 3, parts = min(a.kp, ksteps(0));       // a single short stage may not reach every part
         for (int i = warp >> 2; i < ntile; i += kTThreads / 128) {
             const int R = row0 + i * 128 + q * 32 + lane;
             for (int co0 = 0; co0 < a.Cout; co0 += 16) {
                 float sum[16];
                 tmem_ld16(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(i * a.kp * a.Cout + co0), sum);
-                for (int part = 1; part < a.kp; ++part) {
+                for (int part = 1; part < parts; ++part) {
                     float v[16];
                     tmem_ld16(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)((i * a.kp + part) * a.Cout + co0), v);
 #pragma unroll

@@ -13,7 +13,8 @@ pytestmark = pytest.mark.gpu
 # that reach past the last row or plane, several chunk groups and slices, segments, and the other kernel
 SHAPES = [((1, 1, 16), 16, 16, True), ((3, 5, 32), 48, 16, True), ((9, 9, 32), 96, 32, True), ((6, 7, 80), 32, 96, True),
           ((5, 13, 16), 112, 16, True), ((19, 11, 32), 80, 16, True), ((30, 33, 112), 16, 32, True),
-          ((7, 10, 64), 64, 64, False), ((23, 16, 16), 64, 128, False), ((11, 6, 48), 192, 64, False)]
+          ((7, 10, 64), 64, 64, False), ((23, 16, 16), 64, 128, False), ((11, 6, 48), 192, 64, False),
+          ((5, 13, 16), 64, 64, False)]          # its last stage reaches past the volume
 BAD = (np.nan, np.inf, -np.inf)
 
 
