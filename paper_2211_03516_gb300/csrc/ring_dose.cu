@@ -11,13 +11,14 @@
 //     16-byte vector reductions (groups that are zero are skipped) while the next rows are
 //     walked; gather_turns_kernel adds the four turns up in the caller's layout.
 //
-// Bound by the atomics (53 % of the shared-memory pipe's cycles, 1.64 cycles each: lanes whose
-// rays are less than a voxel apart meet in a bank) and by issue (72 %).  Against the
-// per-angle kernel (operators.cu): 256^3 with 16 jittered rays, 120 angles 122.8 -> 104.8 ms;
-// tall build, BF16, 48 angles 64.4 -> 55.2; large print, 16 angles 93.9 -> 77.1.  Groups of two
-// and single angles share too little of the walk to pay for the run sums (64^3, 90 angles,
-// groups of two: an optimiser iteration 5 % slower; 45 angles: 0.75 -> 1.11 ms): they keep
-// the per-angle kernel.
+// Bound by the shared-memory pipe (95 % of its active cycles with every pixel lit, 1.71 wavefronts per atomic:
+// lanes whose rays are less than a voxel apart meet in a bank; issue 63 %).  Against the per-angle kernel
+// (operators.cu), us, a third to a half of the pixels lit: 256^3 with 16 jittered rays, 120 angles 119479 ->
+// 99765; tall build, BF16, 48 angles 65628 -> 52401; large print, 16 angles 91306 -> 73370.  Four accumulators
+// are cleared and gathered whatever is lit, so a dose of a few pixels takes longer (768 x 768 x 1024 at 16 angles,
+// one pixel lit, 3455 -> 5342).  Groups of two and single angles share too little of the walk to pay for the
+// run sums (64^3, 90 angles, groups of two: an optimiser iteration 5 % slower; 45 angles: 0.75 -> 1.11 ms): they
+// keep the per-angle kernel.
 #include <algorithm>
 #include <type_traits>
 
